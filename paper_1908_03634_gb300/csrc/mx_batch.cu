@@ -98,7 +98,7 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
             return nullptr;
         }
         B->box.push_back(P);
-        const int lc = coarse_start(P->H32);
+        const int lc = coarse_start(P->H32, 0);
         if (lc >= P->H32.nlev) {
             *st = set_err(c, MX_ERR_ARG, "batched: a box has no coarse level of <= 4096 cells (odd sizes too large)");
             free_batch(B);
@@ -201,9 +201,8 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
         dfb[b].part_off = off[b];
         dfb[b].zc = zcs[b];
         const int lc = B->lc[b];
-        coarse_fill_args(cargs.data() + cab * b, &H.lev[lc], H.nlev - lc, o.nu1, o.nu2, o.bottom_iters,
-                         geom_singular(g[b]));
-        B->coarse_smem = std::max(B->coarse_smem, coarse_smem_bytes_f(&H.lev[lc], H.nlev - lc));
+        B->coarse_smem = std::max(B->coarse_smem, coarse_fill_args(cargs.data() + cab * b, &H.lev[lc], H.nlev - lc,
+                                                                   o.nu1, o.nu2, o.bottom_iters, geom_singular(g[b])));
     }
     Bump dry{nullptr, 0};
     auto carve = [&](Bump &bm) {

@@ -190,14 +190,14 @@ void destroy_plans(mx_ctx *c) {
 //    without reading it and the first post-sweep applies the prolongation on
 //    load; the first output buffer is chosen so that the result ends in e;
 //  * other levels above the coarse end: two-pass colour kernels in place;
-//  * the coarse end (levels of <= COARSE_MAX_CELLS cells, down to the bottom):
-//    one single-CTA kernel; without such a level, a BiCGStab bottom kernel.
+//  * the coarse end (the levels that fit one cluster's shared memory, down to the
+//    bottom): one launch; without such a level, a BiCGStab bottom kernel.
 constexpr long long FUSED_MIN_CELLS = 1LL << 18;
 
 template <typename T>
-int coarse_start(const Hier<T> &H) {
+int coarse_start(const Hier<T> &H, int clustered) {
     for (int l = 0; l < H.nlev; l++)
-        if (H.lev[l].g.N <= COARSE_MAX_CELLS && coarse_fits(&H.lev[l], H.nlev - l)) return l;
+        if (coarse_fits(&H.lev[l], H.nlev - l, clustered)) return l;
     return H.nlev;
 }
 
@@ -205,7 +205,7 @@ template <typename T>
 void vcycle(cudaStream_t s, Hier<T> &H, int nu1, int nu2, int bot_iters, int singular, mx_ctx *pc, int fused,
             int zcap) {
     const int nl = H.nlev;
-    const int lc = coarse_start(H);
+    const int lc = coarse_start(H, 1);
     const int ldown = lc < nl ? lc : nl - 1;  // levels with their own kernels
     const bool can_fuse = sizeof(T) == sizeof(float) && fused && nu1 >= 1 && nu2 >= 1;
     auto is_fused = [&](int l) { return can_fuse && H.lev[l].g.N >= FUSED_MIN_CELLS && rbgs_fused_ok(H.lev[l].g); };
@@ -273,7 +273,7 @@ void vcycle(cudaStream_t s, Hier<T> &H, int nu1, int nu2, int bot_iters, int sin
         if (l == 0) prof_end(pc, s, MX_PH_SMOOTH_FINE, is_fused(0) ? nu2 : 1 + 2 * nu2);
     }
 }
-template int coarse_start<float>(const Hier<float> &);
+template int coarse_start<float>(const Hier<float> &, int);
 template void vcycle<float>(cudaStream_t, Hier<float> &, int, int, int, int, mx_ctx *, int, int);
 template void vcycle<double>(cudaStream_t, Hier<double> &, int, int, int, int, mx_ctx *, int, int);
 

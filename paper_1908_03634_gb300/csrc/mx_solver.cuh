@@ -42,7 +42,7 @@ void setup_coefficients(mx_ctx *c, MacPlan &P, const double *rho, const double *
 void setup_coefficients_on(cudaStream_t s, MacPlan &P, const double *rho, const double *beta0);
 mx_status check_opts(mx_ctx *c, const mx_opts *in, mx_opts &o);
 template <typename T>
-int coarse_start(const Hier<T> &H);
+int coarse_start(const Hier<T> &H, int clustered);
 void destroy_plans(mx_ctx *c);
 mx_status ensure_partials(mx_ctx *c, long long nblocks);
 
