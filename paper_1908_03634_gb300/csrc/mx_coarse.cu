@@ -11,10 +11,14 @@
 // side; the owner of a boundary cell stores its update into the neighbour's copy
 // through distributed shared memory, and a cluster barrier ends each colour
 // pass.  Smaller levels run on CTA 0 with block barriers while the other CTAs
-// wait at the next cluster barrier.  The work is latency: a colour pass is six
-// shared loads and a division per cell between two barriers, so the cells'
-// coefficients and neighbour indices are set up once per level visit and the
-// passes touch shared memory only.
+// wait at the next cluster barrier.
+//
+// The work is latency, and above all instruction fetch: a warp runs a level's
+// code once, so code that is not in the instruction cache costs more than the
+// arithmetic.  A thread therefore owns cells of one colour, and the loop over
+// the passes is one short body: six shared loads through precomputed offsets,
+// the update with the coefficients and reciprocal diagonal in registers, a store
+// and a barrier.
 #include <algorithm>
 #include <cstring>
 
@@ -22,20 +26,20 @@
 #include "mx_rbgs.cuh"
 #include "mx_stencil.cuh"
 
-constexpr int CT = 512;          // threads per CTA
-constexpr int BOT_REGS = 3;      // bottom solves of up to BOT_REGS * CT cells keep their vectors in registers
+constexpr int CT = 1024;         // threads per CTA
+constexpr int BOT_REGS = 2;      // bottom solves of up to BOT_REGS * CT cells keep their vectors in registers
 constexpr int COARSE_NC = 16;    // CTAs of the cluster (8 where the device cannot place 16)
 
-// cells per thread of the widest level a CTA may own
-template <typename T>
-struct CoarseCpt {
-    static constexpr int value = sizeof(T) == sizeof(float) ? 8 : 4;
-};
-// levels above this many cells are spread over the cluster (below it one CTA's
-// pass is shorter than a cluster barrier)
+// cells per thread of the widest level a CTA may own, in a cluster and alone
+constexpr int CELLS_CLUSTER = 2, CELLS_ALONE = 4;
+// Levels above this many cells are spread over the cluster.  16^3 on one CTA took
+// 3000 clocks per colour pass (four cells per thread, spilled registers), 1300
+// spread over 8 CTAs, 600 of them the cluster barrier; 8^3 takes 500 on one CTA.
+// FP64 is bound by its pipe (a warp instruction takes about 64 clocks of a
+// quarter of the SM), so it spreads the next level down too.
 template <typename T>
 constexpr int dist_min() {
-    return sizeof(T) == sizeof(float) ? 4096 : 512;
+    return sizeof(T) == sizeof(float) ? 1024 : 512;
 }
 
 // Exact division of x < 2^16 by d < 2^16 as a multiply-high with the
@@ -47,16 +51,17 @@ struct FastDiv {
 inline FastDiv fast_div(unsigned d) { return FastDiv{d, unsigned(((1ull << 32) + d - 1) / d)}; }
 __device__ __forceinline__ int fdiv(int x, FastDiv f) { return f.d == 1 ? x : int(__umulhi(unsigned(x), f.m)); }
 
-// One level of the coarse end.  Shared-memory offsets are in elements and equal
-// in every CTA; the correction holds pp + 2 planes (a neighbour's plane first and
+// One level of the coarse end.  Shared-memory offsets are in bytes and equal in
+// every CTA; the correction holds pp + 2 planes (a neighbour's plane first and
 // last), the right-hand side pp planes.
 template <typename T>
 struct CoarseLevel {
     Level<T> L;
-    FastDiv d0, d1, dh;  // n0, n1, n0 / 2
+    FastDiv d0, d1, dh, dp;  // n0, n1, n0 / 2, pp
     int dist;            // spread over the cluster
     int pp;              // planes per CTA (even where dist)
     int eoff, foff;
+    T h2, ih2;           // h^2 and 1 / h^2, rounded as the other kernels round them
 };
 
 template <typename T>
@@ -66,471 +71,358 @@ struct CoarseArgs {
     int nu1, nu2, bot_iters, singular;
     int nc;    // CTAs
     int roff;  // scratch: the residuals of a level, then the bottom solve's vectors
-    int total; // elements of shared memory
+    int total; // bytes of shared memory
 };
+
+extern __shared__ __align__(16) unsigned char coarse_smem[];
+template <typename T>
+__device__ __forceinline__ T &sm_at(int byte) {
+    return *reinterpret_cast<T *>(coarse_smem + byte);
+}
 
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-__device__ __forceinline__ unsigned cluster_addr(const void *p, int rank) {
-    unsigned a = unsigned(__cvta_generic_to_shared(p)), r;
+// address of this CTA's shared byte in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned cluster_addr(int byte, int rank) {
+    const unsigned a = unsigned(__cvta_generic_to_shared(coarse_smem)) + byte;
+    unsigned r;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void remote_store(float *p, int rank, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "f"(v) : "memory");
+__device__ __forceinline__ void remote_store(unsigned a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
-__device__ __forceinline__ void remote_store(double *p, int rank, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "d"(v) : "memory");
+__device__ __forceinline__ void remote_store(unsigned a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
-__device__ __forceinline__ float remote_load(const float *p, int rank) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
-    return v;
+__device__ __forceinline__ void remote_load(unsigned a, float &v) {
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
 }
-__device__ __forceinline__ double remote_load(const double *p, int rank) {
-    double v;
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(cluster_addr(p, rank)) : "memory");
-    return v;
+__device__ __forceinline__ void remote_load(unsigned a, double &v) {
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
 }
-__device__ __forceinline__ void level_sync(int dist) {
+
+// The threads that hold a level's cells: the cluster, or the block's first nthr
+// threads (whole warps; a small level's barriers then cost less).
+__device__ __forceinline__ void team_sync(int dist, int nthr) {
     if (dist) cluster_sync();
-    else __syncthreads();
+    else asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
 }
-
-// The part of a level a CTA owns, and where its boundary planes are copied to.
-struct Slab {
-    int k0, np;          // first plane, planes
-    int dn, up;          // ranks holding copies of the first / last plane (-1: none)
-    int dn_plane;        // plane of dn's buffer that copies this CTA's first plane
-    int dist;
-};
-
-template <typename T>
-__device__ __forceinline__ Slab slab_of(const CoarseLevel<T> &C, int rank) {
-    Slab s;
-    const int nz = C.L.g.n[2];
-    const bool per = gper(C.L.g, 2);
-    s.dist = C.dist;
-    s.k0 = rank * C.pp;
-    s.np = max(0, min(C.pp, nz - s.k0));
-    const int last = (nz - 1) / C.pp;
-    const bool first_here = rank == 0, last_here = rank == last;
-    s.dn = first_here ? (per ? last : -1) : rank - 1;
-    s.up = last_here ? (per ? 0 : -1) : rank + 1;
-    s.dn_plane = (s.dn == last ? nz - last * C.pp : C.pp) + 1;
-    return s;
-}
-
-// The cells of one thread: coefficients, own index and neighbour indices in the
-// shared correction.  Slots [0, CPT/2) hold red cells, the rest black ones.
-template <typename T, int CPT>
-struct Cells {
-    T b[CPT][6];
-    T inv[CPT];            // FP64: 1 / sum of b
-    unsigned xn[CPT];      // x neighbours (low half: i - 1)
-    unsigned yn[CPT];      // y neighbours
-    int at[CPT];           // own index; -1: no cell
-};
 
 // the 6 face coefficients of in-box cell (i,j,k) = c with 32-bit indexing (the
-// same values as face_coefs)
+// same values as face_coefs); addresses are selected, so the loads issue together
 template <typename T>
 __device__ __forceinline__ void coefs32(const Level<T> &L, int i, int j, int k, int c, T b[6]) {
     const DGeom &g = L.g;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxy = nx * ny;
-    const bool px = gper(g, 0), py = gper(g, 1), pz = gper(g, 2);
+    const bool hx = i + 1 == nx && !gper(g, 0), hy = j + 1 == ny && !gper(g, 1), hz = k + 1 == nz && !gper(g, 2);
+    const T *px = hx ? L.hx : L.bx, *py = hy ? L.hy : L.by, *pz = hz ? L.hz : L.bz;
+    const int ox = hx ? j + ny * k : (i + 1 == nx ? c - (nx - 1) : c + 1);
+    const int oy = hy ? i + nx * k : (j + 1 == ny ? c - (ny - 1) * nx : c + nx);
+    const int oz = hz ? i + nx * j : (k + 1 == nz ? c - (nz - 1) * nxy : c + nxy);
     b[0] = L.bx[c];
-    b[1] = (i + 1 < nx) ? L.bx[c + 1] : (px ? L.bx[c - (nx - 1)] : L.hx[j + ny * k]);
+    b[1] = px[ox];
     b[2] = L.by[c];
-    b[3] = (j + 1 < ny) ? L.by[c + nx] : (py ? L.by[c - (ny - 1) * nx] : L.hy[i + nx * k]);
+    b[3] = py[oy];
     b[4] = L.bz[c];
-    b[5] = (k + 1 < nz) ? L.bz[c + nxy] : (pz ? L.bz[c - (nz - 1) * nxy] : L.hz[i + nx * j]);
+    b[5] = pz[oz];
 }
 
-// Index 0 of the shared array holds 0: the neighbour beyond a non-periodic face.
-template <typename T, int CPT>
-__device__ __forceinline__ void load_cells(const CoarseLevel<T> &C, const Slab &s, Cells<T, CPT> &R) {
+// The cells of one thread, all of one colour: coefficients and shared offsets.
+template <typename T, int SL>
+struct Cells {
+    T b[SL][6];
+    T inv[SL];        // 1 / sum of b
+    int at[SL];       // the cell's correction; 0: no cell
+    unsigned xn[SL];  // its x neighbours (low half: i - 1), y neighbours
+    unsigned yn[SL];
+    unsigned push[SL];  // cluster address of the copy of it (0: none)
+};
+
+template <typename T, int SL>
+__device__ __forceinline__ void neighbours(const Cells<T, SL> &R, int q, int plane, T v[6]) {
+    v[0] = sm_at<T>(R.xn[q] & 0xffffu);
+    v[1] = sm_at<T>(R.xn[q] >> 16);
+    v[2] = sm_at<T>(R.yn[q] & 0xffffu);
+    v[3] = sm_at<T>(R.yn[q] >> 16);
+    v[4] = sm_at<T>(R.at[q] - plane);
+    v[5] = sm_at<T>(R.at[q] + plane);
+}
+
+// One level on the way down (smoothing from e = 0, restriction to the level
+// below) or up (prolongation, smoothing), with SL cells per thread.
+template <typename T, int SL>
+__device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, bool up) {
+    constexpr int B = sizeof(T);
+    const CoarseLevel<T> &C = A.lev[l], &F = A.lev[l + 1];
     const DGeom &g = C.L.g;
-    const int nx = g.n[0], ny = g.n[1], nxy = nx * ny, half = (nxy * s.np) >> 1;
-    const bool px = gper(g, 0), py = gper(g, 1);
+    const int nx = g.n[0], ny = g.n[1], nxy = nx * ny, dist = C.dist;
+    const int k0 = rank * C.pp, np = max(0, min(C.pp, g.n[2] - k0)), half = (nxy * np) >> 1;
+    const int team = dist ? CT / 2 : ((half + SL - 1) / SL + 31) & ~31;  // threads per colour
+    if (int(threadIdx.x) >= 2 * team) return;
+    const int colour = int(threadIdx.x) >= team;
+    const int e0 = C.eoff + nxy * B, plane = nxy * B, df = C.foff - e0;
+    Cells<T, SL> R;
+    {
+        // ranks that hold copies of the first and the last plane (-1: none)
+        const bool px = gper(g, 0), py = gper(g, 1), pz = gper(g, 2);
+        const int last = (g.n[2] - 1) / C.pp;
+        const int dn = rank > 0 ? rank - 1 : (pz ? last : -1), upr = rank < last ? rank + 1 : (pz ? 0 : -1);
+        const int dnp = dn == last ? g.n[2] - last * C.pp : C.pp;  // dn's planes
 #pragma unroll
-    for (int q = 0; q < CPT; q++) {
-        const int colour = q >= CPT / 2;
-        const int m = threadIdx.x + CT * (q % (CPT / 2));
-        R.at[q] = -1;
-        if (m < half) {
-            const int r = fdiv(m, C.dh);  // row j + n1 p
-            const int p = fdiv(r, C.d1);
-            const int j = r - p * ny, k = s.k0 + p;
-            const int i = 2 * (m - r * int(C.dh.d)) + ((j + k + colour) & 1);
-            coefs32(C.L, i, j, k, i + nx * (j + ny * k), R.b[q]);
-            const int a = C.eoff + nxy + i + nx * r;
-            R.at[q] = a;
-            const int xl = i > 0 ? a - 1 : (px ? a + nx - 1 : 0), xh = i + 1 < nx ? a + 1 : (px ? a - (nx - 1) : 0);
-            const int yl = j > 0 ? a - nx : (py ? a + (ny - 1) * nx : 0);
-            const int yh = j + 1 < ny ? a + nx : (py ? a - (ny - 1) * nx : 0);
-            R.xn[q] = unsigned(xl) | (unsigned(xh) << 16);
-            R.yn[q] = unsigned(yl) | (unsigned(yh) << 16);
-            if (sizeof(T) == sizeof(double)) {
-                const T *b = R.b[q];
-                R.inv[q] = T(1) / ((b[0] + b[1]) + (b[2] + b[3]) + (b[4] + b[5]));
+        for (int q = 0; q < SL; q++) {
+            const int m = int(threadIdx.x) - colour * team + team * q;
+            R.at[q] = 0;
+            R.push[q] = 0;
+            if (m < half) {
+                const int r = fdiv(m, C.dh);  // row j + n1 p
+                const int p = fdiv(r, C.d1);
+                const int j = r - p * ny, k = k0 + p;
+                const int i = 2 * (m - r * int(C.dh.d)) + ((j + k + colour) & 1);
+                coefs32(C.L, i, j, k, i + nx * (j + ny * k), R.b[q]);
+                const int a = e0 + (i + nx * r) * B;
+                R.at[q] = a;
+                // offset 0 holds 0: the neighbour beyond a non-periodic face
+                const int xl = i > 0 ? a - B : (px ? a + (nx - 1) * B : 0);
+                const int xh = i + 1 < nx ? a + B : (px ? a - (nx - 1) * B : 0);
+                const int yl = j > 0 ? a - nx * B : (py ? a + (ny - 1) * nx * B : 0);
+                const int yh = j + 1 < ny ? a + nx * B : (py ? a - (ny - 1) * nx * B : 0);
+                R.xn[q] = unsigned(xl) | (unsigned(xh) << 16);
+                R.yn[q] = unsigned(yl) | (unsigned(yh) << 16);
+                const int in_plane = (i + nx * j) * B;
+                if (p == 0 && dn >= 0) R.push[q] = cluster_addr(C.eoff + (dnp + 1) * plane + in_plane, dn);
+                if (p == np - 1 && upr >= 0) R.push[q] = cluster_addr(C.eoff + in_plane, upr);
+                if constexpr (B == 4) R.inv[q] = gs_inverse(R.b[q]);
+                else R.inv[q] = C.L.di[i + nx * (j + ny * k)];
             }
         }
     }
-}
-
-template <typename T, int CPT>
-__device__ __forceinline__ void neighbours(const T *sm, const Cells<T, CPT> &R, int q, int nxy, T v[6]) {
-    v[0] = sm[R.xn[q] & 0xffffu];
-    v[1] = sm[R.xn[q] >> 16];
-    v[2] = sm[R.yn[q] & 0xffffu];
-    v[3] = sm[R.yn[q] >> 16];
-    v[4] = sm[R.at[q] - nxy];
-    v[5] = sm[R.at[q] + nxy];
-}
-
-// store cell `a`'s new value, and into the copies of it
-template <typename T>
-__device__ __forceinline__ void put(T *sm, int eoff, const Slab &s, int nxy, int a, T v) {
-    sm[a] = v;
-    const int ji = a - eoff - nxy;  // index within the slab
-    if (ji < nxy && s.dn >= 0) {
-        T *t = sm + eoff + s.dn_plane * nxy + ji;
-        if (s.dist) remote_store(t, s.dn, v);
-        else *t = v;
-    }
-    if (ji >= (s.np - 1) * nxy && s.up >= 0) {
-        T *t = sm + eoff + ji - (s.np - 1) * nxy;
-        if (s.dist) remote_store(t, s.up, v);
-        else *t = v;
-    }
-}
-
-// FP32: the same rounded operations as gs_update (bit for bit); FP64: the
-// division as a product with the reciprocal taken once per level visit.
-__device__ __forceinline__ float cell_update(const float b[6], const float v[6], float f, float h2, float) {
-    return gs_update(b, v, f, h2);
-}
-__device__ __forceinline__ double cell_update(const double b[6], const double v[6], double f, double h2, double inv) {
-    double num = b[0] * v[0];
-    for (int q = 1; q < 6; q++) num = fma(b[q], v[q], num);
-    return fma(-h2, f, num) * inv;
-}
-
-template <typename T, int CPT>
-__device__ __forceinline__ void sweeps(T *sm, const CoarseLevel<T> &C, const Slab &s, const Cells<T, CPT> &R, int nu) {
-    const int nxy = int(C.L.g.nxy), df = C.foff - C.eoff - nxy;
-    const T h2 = T(C.L.g.h * C.L.g.h);
-    for (int w = 0; w < nu; w++) {
+    if (up) {  // e += the parents' corrections
+        const int mx = nx >> 1, mxy = nxy >> 2;
 #pragma unroll
-        for (int colour = 0; colour < 2; colour++) {
-            T e[CPT / 2];
+        for (int q = 0; q < SL; q++)
+            if (R.at[q]) {
+                const int c = (R.at[q] - e0) / B;
+                const int r = fdiv(c, C.d0);
+                const int p = fdiv(r, C.d1);
+                const int i = c - r * nx, j = r - p * ny, K = (k0 + p) >> 1;
+                const int owner = F.dist ? fdiv(K, F.dp) : 0;
+                const int src = F.eoff + (mxy + (i >> 1) + mx * (j >> 1) + mxy * (K - owner * F.pp)) * B;
+                T ec;
+                if (dist) remote_load(cluster_addr(src, owner), ec);
+                else ec = sm_at<T>(src);
+                const T v = sm_at<T>(R.at[q]) + ec;
+                sm_at<T>(R.at[q]) = v;
+                if (R.push[q]) remote_store(R.push[q], v);
+            }
+        team_sync(dist, 2 * team);
+    }
+    const T h2 = C.h2;
+    const int passes = 2 * (up ? A.nu2 : A.nu1);
+#pragma unroll 1
+    for (int w = 0; w < passes; w++) {
+        if ((w & 1) == colour) {
 #pragma unroll
-            for (int h = 0; h < CPT / 2; h++) {
-                const int q = colour * (CPT / 2) + h;
-                if (R.at[q] >= 0) {
+            for (int q = 0; q < SL; q++)
+                if (R.at[q]) {
                     T v[6];
-                    neighbours(sm, R, q, nxy, v);
-                    e[h] = cell_update(R.b[q], v, sm[R.at[q] + df], h2, R.inv[q]);
+                    neighbours(R, q, plane, v);
+                    const T e = gs_update(R.b[q], v, sm_at<T>(R.at[q] + df), h2, R.inv[q]);
+                    sm_at<T>(R.at[q]) = e;
+                    if (R.push[q]) remote_store(R.push[q], e);
                 }
-            }
+        }
+        team_sync(dist, 2 * team);
+    }
+    if (!up) {  // the level below: right-hand side = means of the 8 residuals
+        const T ih2 = C.ih2;
 #pragma unroll
-            for (int h = 0; h < CPT / 2; h++) {
-                const int q = colour * (CPT / 2) + h;
-                if (R.at[q] >= 0) put(sm, C.eoff, s, nxy, R.at[q], e[h]);
+        for (int q = 0; q < SL; q++)
+            if (R.at[q]) {
+                T v[6];
+                neighbours(R, q, plane, v);
+                sm_at<T>(A.roff + R.at[q] - e0) =
+                    sm_at<T>(R.at[q] + df) - flux_sum(R.b[q], v, sm_at<T>(R.at[q])) * ih2;
             }
-            level_sync(s.dist);
-        }
-    }
-}
-
-// residual of level C restricted to the right-hand side of F, the next one
-template <typename T, int CPT>
-__device__ __forceinline__ void restrict_down(T *sm, const CoarseArgs<T> &A, const CoarseLevel<T> &C,
-                                              const CoarseLevel<T> &F, const Slab &s, const Cells<T, CPT> &R) {
-    const int nx = C.L.g.n[0], nxy = int(C.L.g.nxy), df = C.foff - C.eoff - nxy;
-    const T ih2 = T(1) / T(C.L.g.h * C.L.g.h);
-    T *rs = sm + A.roff;
+        team_sync(0, 2 * team);
+        const int mx = nx >> 1, mxy = nxy >> 2, nown = (nxy * np) >> 3;
+        for (int t = threadIdx.x; t < nown; t += 2 * team) {
+            const int r = fdiv(t, F.d0);
+            const int P = fdiv(r, F.d1);
+            const int I = t - r * mx, J = r - P * int(F.d1.d), K = (k0 >> 1) + P;
+            const int c = A.roff + (2 * I + nx * (2 * J) + nxy * (2 * P)) * B;
+            T sum = T(0);
 #pragma unroll
-    for (int q = 0; q < CPT; q++)
-        if (R.at[q] >= 0) {
-            T v[6];
-            neighbours(sm, R, q, nxy, v);
-            rs[R.at[q] - C.eoff - nxy] = sm[R.at[q] + df] - flux_sum(R.b[q], v, sm[R.at[q]]) * ih2;
-        }
-    __syncthreads();
-    const int mx = nx >> 1, mxy = nxy >> 2, nown = (nxy * s.np) >> 3;
-    for (int t = threadIdx.x; t < nown; t += CT) {
-        const int r = fdiv(t, F.d0);
-        const int P = fdiv(r, F.d1);
-        const int I = t - r * mx, J = r - P * int(F.d1.d), K = (s.k0 >> 1) + P;
-        const T *c = rs + 2 * I + nx * (2 * J) + nxy * (2 * P);
-        T sum = T(0);
-        for (int dk = 0; dk < 2; dk++)
-            for (int dj = 0; dj < 2; dj++)
-                for (int di = 0; di < 2; di++) sum += c[di + nx * dj + nxy * dk];
-        const int owner = F.dist ? K / F.pp : 0;
-        T *dst = sm + F.foff + I + mx * J + mxy * (K - owner * F.pp);
-        if (s.dist) remote_store(dst, owner, sum * T(0.125));
-        else *dst = sum * T(0.125);
-    }
-    level_sync(s.dist);
-}
-
-// e += the parents' corrections
-template <typename T, int CPT>
-__device__ __forceinline__ void prolong_up(T *sm, const CoarseLevel<T> &C, const CoarseLevel<T> &F, const Slab &s,
-                                           const Cells<T, CPT> &R) {
-    const int nx = C.L.g.n[0], nxy = int(C.L.g.nxy), mx = nx >> 1, mxy = nxy >> 2;
-#pragma unroll
-    for (int q = 0; q < CPT; q++)
-        if (R.at[q] >= 0) {
-            const int r = fdiv(R.at[q] - C.eoff - nxy, C.d0);
-            const int p = fdiv(r, C.d1);
-            const int i = R.at[q] - C.eoff - nxy - r * nx, j = r - p * int(C.d1.d), K = (s.k0 + p) >> 1;
-            const int owner = F.dist ? K / F.pp : 0;
-            const T *src = sm + F.eoff + mxy + (i >> 1) + mx * (j >> 1) + mxy * (K - owner * F.pp);
-            const T ec = s.dist ? remote_load(src, owner) : *src;
-            put(sm, C.eoff, s, nxy, R.at[q], sm[R.at[q]] + ec);
-        }
-    level_sync(s.dist);
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// BiCGStab on a bottom level of at most 32 cells by one warp: one cell per
-// lane, dot products by shuffles, the operator's neighbour values through a
-// shared-memory vector; no block barriers.
-template <typename T>
-__device__ void warp_bicgstab(const Level<T> &L, T *x, const T *f, T *pv, int iters, int singular, T ih2) {
-    const int n = int(L.g.N), lane = threadIdx.x;
-    const bool act = lane < n;
-    int i = 0, j = 0, k = 0;
-    T b[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    if (act) {
-        i = lane % L.g.n[0];
-        const int r = lane / L.g.n[0];
-        j = r % L.g.n[1];
-        k = r / L.g.n[1];
-        face_coefs(L, i, j, k, lane, b);
-    }
-    auto apply = [&](T val) -> T {  // (L val)_lane, values exchanged through pv
-        if (act) pv[lane] = val;
-        __syncwarp();
-        T y = T(0);
-        if (act) {
-            T v[6];
-            nb_vals(L.g, (const T *)pv, i, j, k, lane, v);
-            y = flux_sum(b, v, val) * ih2;
-        }
-        __syncwarp();
-        return y;
-    };
-    T rhs = act ? f[lane] : T(0);
-    if (singular) rhs -= warp_sum(rhs) / T(n);
-    if (!act) rhs = T(0);
-    T xv = T(0), r = rhs, r0 = rhs, p = T(0), v = T(0);
-    const T bnorm2 = warp_sum(rhs * rhs);
-    if (bnorm2 > T(0)) {
-        const T tol2 = bnorm2 * T(1e-8);
-        T rho = T(1), alpha = T(1), omega = T(1);
-        for (int it = 0; it < iters; it++) {
-            const T rho1 = warp_sum(r0 * r);
-            if (rho1 == T(0) || omega == T(0)) break;
-            const T beta = (rho1 / rho) * (alpha / omega);
-            p = r + beta * (p - omega * v);
-            v = apply(p);
-            const T r0v = warp_sum(r0 * v);
-            if (r0v == T(0)) break;
-            alpha = rho1 / r0v;
-            const T sv = r - alpha * v;
-            if (warp_sum(sv * sv) <= tol2) {
-                xv += alpha * p;
-                break;
-            }
-            const T tv = apply(sv);
-            const T tt = warp_sum(tv * tv), ts = warp_sum(tv * sv);
-            omega = tt > T(0) ? ts / tt : T(0);
-            xv += alpha * p + omega * sv;
-            r = sv - omega * tv;
-            rho = rho1;
-            if (warp_sum(r * r) <= tol2) break;
+            for (int d = 0; d < 8; d++)
+                sum += sm_at<T>(c + ((d & 1) + nx * ((d >> 1) & 1) + nxy * (d >> 2)) * B);
+            const int owner = F.dist ? fdiv(K, F.dp) : 0;
+            const int dst = F.foff + (I + mx * J + mxy * (K - owner * F.pp)) * B;
+            if (dist) remote_store(cluster_addr(dst, owner), sum * T(0.125));
+            else sm_at<T>(dst) = sum * T(0.125);
         }
     }
-    if (!act) xv = T(0);
-    if (singular) xv -= warp_sum(xv) / T(n);
-    if (act) x[lane] = xv;
 }
 
-// Sums of three values over the first nthr threads of the block (whole warps),
-// in every one of them: warp shuffles, then each warp adds the warps' sums
-// itself.  The two buffers alternate, so one barrier separates the writes of a
-// reduction from those of the next but one.
-template <typename T>
-__device__ __forceinline__ void team_sum3(T &a, T &b, T &c, T (*red)[3][32], int &turn, int nthr) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = nthr >> 5;
-    a = warp_sum(a);
-    b = warp_sum(b);
-    c = warp_sum(c);
-    T(*buf)[32] = red[turn];
-    turn ^= 1;
-    if (lane == 0) {
-        buf[0][w] = a;
-        buf[1][w] = b;
-        buf[2][w] = c;
-    }
-    asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-    a = lane < nw ? buf[0][lane] : T(0);
-    b = lane < nw ? buf[1][lane] : T(0);
-    c = lane < nw ? buf[2][lane] : T(0);
-    for (int o = 8; o > 0; o >>= 1) {  // nw <= 16
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    a = __shfl_sync(0xffffffffu, a, 0);
-    b = __shfl_sync(0xffffffffu, b, 0);
-    c = __shfl_sync(0xffffffffu, c, 0);
-}
+// The bottom solve's scalar divisions: they set its step lengths, so the fast
+// forms (a subroutine's instructions would cost more than its arithmetic).
+__device__ __forceinline__ float sdiv(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b); }
 
 // BiCGStab on L x = f (x starts at 0), projected onto mean-free vectors when
 // the problem is singular; stops at relative residual 1e-4 or `iters`.  Each of
-// nthr threads holds up to B cells (cell t + q nthr): their coefficients and all
-// vectors stay in registers, the two vectors the operator is applied to pass
-// through shared memory (element n holds 0 for faces without a neighbour), and
-// the reductions that one step needs are taken together: five barriers per
-// iteration.
+// nthr threads (whole warps) holds up to B cells (cell t + q nthr): coefficients
+// and vectors stay in registers, and the vector the operator is applied to passes
+// through shared memory (element n holds 0 for faces without a neighbour).
+//
+// The cost is instruction fetch and the latency of the sums, so the iteration is
+// one rolled body run twice (v = L p, t = L s) with one reduction each:
+//   r0.v gives alpha; s.s, t.t, t.s and r0.t give omega, the next residual's norm
+//   s.s - 2 omega t.s + omega^2 t.t, and the next r0.r = -omega r0.t, since
+//   r0.s = r0.r - alpha r0.v = 0.
+// The operations are rounded explicitly, so the single and the batched kernel
+// agree bit for bit.
 template <typename T, int B>
-__device__ void team_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular, T ih2, int nthr) {
-    __shared__ T red[2][3][32];
+__device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular,
+                                              T ih2, int nthr) {
+    __shared__ T red[2][4][32];
     const int n = int(L.g.N), nx = L.g.n[0], ny = L.g.n[1], nz = L.g.n[2], nxy = nx * ny;
-    const bool px = gper(L.g, 0), py = gper(L.g, 1), pz = gper(L.g, 2);
-    T *pe = scr, *se = scr + n + 1;
-    int turn = 0;
-    T b[B][6], xv[B], r[B], r0[B], p[B], v[B], sv[B], tv[B];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nthr >> 5;
+    T b[B][6], den[B], xv[B], r[B], r0[B], p[B], v[B];
     unsigned nb[B][3];
-    T z0 = T(0), z1 = T(0), sum = T(0);
-    if (threadIdx.x == 0) pe[n] = se[n] = T(0);
+    if (threadIdx.x < 2) scr[threadIdx.x * (n + 1) + n] = T(0);
+    T a[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
     for (int q = 0; q < B; q++) {
         const int c = threadIdx.x + q * nthr;
-        xv[q] = r[q] = p[q] = v[q] = sv[q] = tv[q] = T(0);
+        xv[q] = r[q] = p[q] = v[q] = T(0);
         for (int d = 0; d < 6; d++) b[q][d] = T(0);
         nb[q][0] = nb[q][1] = nb[q][2] = unsigned(n) | (unsigned(n) << 16);
         if (c < n) {
             const int i = c % nx, rr = c / nx, j = rr % ny, k = rr / ny;
+            const bool px = gper(L.g, 0), py = gper(L.g, 1), pz = gper(L.g, 2);
             coefs32(L, i, j, k, c, b[q]);
             const int xl = i > 0 ? c - 1 : (px ? c + nx - 1 : n), xh = i + 1 < nx ? c + 1 : (px ? c - (nx - 1) : n);
-            const int yl = j > 0 ? c - nx : (py ? c + (ny - 1) * nx : n), yh = j + 1 < ny ? c + nx : (py ? c - (ny - 1) * nx : n);
-            const int zl = k > 0 ? c - nxy : (pz ? c + (nz - 1) * nxy : n), zh = k + 1 < nz ? c + nxy : (pz ? c - (nz - 1) * nxy : n);
+            const int yl = j > 0 ? c - nx : (py ? c + (ny - 1) * nx : n);
+            const int yh = j + 1 < ny ? c + nx : (py ? c - (ny - 1) * nx : n);
+            const int zl = k > 0 ? c - nxy : (pz ? c + (nz - 1) * nxy : n);
+            const int zh = k + 1 < nz ? c + nxy : (pz ? c - (nz - 1) * nxy : n);
             nb[q][0] = unsigned(xl) | (unsigned(xh) << 16);
             nb[q][1] = unsigned(yl) | (unsigned(yh) << 16);
             nb[q][2] = unsigned(zl) | (unsigned(zh) << 16);
             r[q] = f[c];
-            sum += r[q];
+            a[0] += r[q];
         }
+        den[q] = radd(radd(radd(b[q][0], b[q][1]), radd(b[q][2], b[q][3])), radd(b[q][4], b[q][5]));
     }
-    auto apply = [&](const T *e, const T(&own)[B], T(&y)[B]) {
+    auto barrier = [&] { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); };
+    // Sums of a[0..4) over the team, the same bits in every thread.  The four sums
+    // share the shuffles (each exchange halves what a lane still carries: 6 in
+    // place of 20), lane group g = lane / 8 ends with sum g.  The two buffers
+    // alternate: a barrier lies between a reduction's reads and the writes of the
+    // next but one.
+    int turn = 0;
+    auto group_sum = [&](T k) {
 #pragma unroll
-        for (int q = 0; q < B; q++) {
-            T w[6];
-            for (int d = 0; d < 3; d++) {
-                w[2 * d] = e[nb[q][d] & 0xffffu];
-                w[2 * d + 1] = e[nb[q][d] >> 16];
-            }
-            y[q] = flux_sum(b[q], w, own[q]) * ih2;
+        for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+        return k;
+    };
+    auto team_sum = [&]() {
+        const bool up16 = lane & 16, up8 = lane & 8;
+        T k0 = up16 ? a[2] : a[0], k1 = up16 ? a[3] : a[1];
+        k0 += __shfl_xor_sync(0xffffffffu, up16 ? a[0] : a[2], 16);
+        k1 += __shfl_xor_sync(0xffffffffu, up16 ? a[1] : a[3], 16);
+        T k = (up8 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up8 ? k0 : k1, 8);
+        k = group_sum(k);
+        if (nw > 1) {
+            if ((lane & 7) == 0) red[turn][lane >> 3][warp] = k;
+            barrier();
+            k = T(0);
+            for (int q = lane & 7; q < nw; q += 8) k += red[turn][lane >> 3][q];
+            k = group_sum(k);
+            turn ^= 1;
         }
-    };
-    auto share = [&](T *e, const T(&own)[B]) {
 #pragma unroll
-        for (int q = 0; q < B; q++)
-            if (threadIdx.x + q * nthr < n) e[threadIdx.x + q * nthr] = own[q];
-        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+        for (int m = 0; m < 4; m++) a[m] = __shfl_sync(0xffffffffu, k, 8 * m);
     };
-    if (singular) {
-        team_sum3(sum, z0, z1, red, turn, nthr);
-        const T mean = sum / T(n);
-#pragma unroll
-        for (int q = 0; q < B; q++)
-            if (threadIdx.x + q * nthr < n) r[q] -= mean;
-    }
-    T rho1 = T(0);
+    const T inv_n = T(1) / T(n);
+    T mean = T(0), rho1 = T(0), rho = T(1), alpha = T(1), omega = T(1), tol2 = T(0);
+    // step -1: the mean of f and ||f - mean||^2; then the iterations
+    team_sum();
+    if (singular) mean = a[0] * inv_n;
+    a[0] = a[1] = a[2] = a[3] = T(0);
 #pragma unroll
     for (int q = 0; q < B; q++) {
+        if (int(threadIdx.x) + q * nthr < n) r[q] -= mean;
         r0[q] = r[q];
-        rho1 += r[q] * r[q];
+        a[0] = rfma(r[q], r[q], a[0]);
     }
-    z0 = z1 = T(0);
-    team_sum3(rho1, z0, z1, red, turn, nthr);
-    const T bnorm2 = rho1;
-    if (bnorm2 > T(0)) {
-        const T tol2 = bnorm2 * T(1e-8);  // 1e-4 relative: ample for a multigrid bottom solve
-        T rho = T(1), alpha = T(1), omega = T(1);
+    team_sum();
+    rho1 = a[0];
+    if (rho1 > T(0)) {
+        tol2 = rho1 * T(1e-8);  // 1e-4 relative: ample for a multigrid bottom solve
+#pragma unroll 1
         for (int it = 0; it < iters; it++) {
             if (rho1 == T(0) || omega == T(0)) break;
-            const T beta = (rho1 / rho) * (alpha / omega);
+            const T beta = sdiv(rho1 * alpha, rho * omega);
+            T w[B], y[B];
 #pragma unroll
-            for (int q = 0; q < B; q++) p[q] = r[q] + beta * (p[q] - omega * v[q]);
-            share(pe, p);
-            apply(pe, p, v);
-            T r0v = T(0);
+            for (int q = 0; q < B; q++) w[q] = p[q] = rfma(beta, rfma(-omega, v[q], p[q]), r[q]);
+            bool stop = false;
+#pragma unroll 1
+            for (int h = 0; h < 2; h++) {  // y = L w: v = L p, then t = L s
+                T *e = scr + h * (n + 1);
 #pragma unroll
-            for (int q = 0; q < B; q++) r0v += r0[q] * v[q];
-            z0 = z1 = T(0);
-            team_sum3(r0v, z0, z1, red, turn, nthr);
-            if (r0v == T(0)) break;
-            alpha = rho1 / r0v;
+                for (int q = 0; q < B; q++)
+                    if (int(threadIdx.x) + q * nthr < n) e[threadIdx.x + q * nthr] = w[q];
+                barrier();
+                a[0] = a[1] = a[2] = a[3] = T(0);
 #pragma unroll
-            for (int q = 0; q < B; q++) sv[q] = r[q] - alpha * v[q];
-            share(se, sv);
-            apply(se, sv, tv);
-            T ss = T(0), tt = T(0), ts = T(0);
+                for (int q = 0; q < B; q++) {
+                    const T s0 = rfma(b[q][0], e[nb[q][0] & 0xffffu], rmul(b[q][1], e[nb[q][0] >> 16]));
+                    const T s1 = rfma(b[q][2], e[nb[q][1] & 0xffffu], rmul(b[q][3], e[nb[q][1] >> 16]));
+                    const T s2 = rfma(b[q][4], e[nb[q][2] & 0xffffu], rmul(b[q][5], e[nb[q][2] >> 16]));
+                    y[q] = rmul(rfma(-den[q], w[q], radd(radd(s0, s1), s2)), ih2);
+                    a[0] = rfma(r0[q], y[q], a[0]);
+                    a[1] = rfma(w[q], w[q], a[1]);
+                    a[2] = rfma(y[q], y[q], a[2]);
+                    a[3] = rfma(y[q], w[q], a[3]);
+                }
+                team_sum();
+                if (h == 0) {
+                    stop = a[0] == T(0);
+                    if (stop) break;
+                    alpha = sdiv(rho1, a[0]);
+#pragma unroll
+                    for (int q = 0; q < B; q++) {
+                        v[q] = y[q];
+                        w[q] = rfma(-alpha, y[q], r[q]);
+                    }
+                }
+            }
+            if (stop) break;
+            const bool small = a[1] <= tol2;  // s is small enough: no second half step
+            omega = !small && a[2] > T(0) ? sdiv(a[3], a[2]) : T(0);
 #pragma unroll
             for (int q = 0; q < B; q++) {
-                ss += sv[q] * sv[q];
-                tt += tv[q] * tv[q];
-                ts += tv[q] * sv[q];
+                xv[q] = rfma(omega, w[q], rfma(alpha, p[q], xv[q]));
+                r[q] = rfma(-omega, y[q], w[q]);
             }
-            team_sum3(ss, tt, ts, red, turn, nthr);
-            if (ss <= tol2) {
-#pragma unroll
-                for (int q = 0; q < B; q++) xv[q] += alpha * p[q];
-                break;
-            }
-            omega = tt > T(0) ? ts / tt : T(0);
-            T rr = T(0), rn = T(0);
-#pragma unroll
-            for (int q = 0; q < B; q++) {
-                xv[q] += alpha * p[q] + omega * sv[q];
-                r[q] = sv[q] - omega * tv[q];
-                rr += r[q] * r[q];
-                rn += r0[q] * r[q];
-            }
+            if (small || rfma(-omega, rfma(-omega, a[2], rmul(T(2), a[3])), a[1]) <= tol2) break;
             rho = rho1;
-            z0 = T(0);
-            team_sum3(rr, rn, z0, red, turn, nthr);
-            if (rr <= tol2) break;
-            rho1 = rn;
+            rho1 = -omega * a[0];
         }
     }
+    a[0] = a[1] = a[2] = a[3] = T(0);
     if (singular) {
-        sum = T(0);
 #pragma unroll
-        for (int q = 0; q < B; q++) sum += xv[q];
-        z0 = z1 = T(0);
-        team_sum3(sum, z0, z1, red, turn, nthr);
-        const T mean = sum / T(n);
-#pragma unroll
-        for (int q = 0; q < B; q++) xv[q] -= mean;
+        for (int q = 0; q < B; q++) a[0] += xv[q];
+        team_sum();
+        mean = a[0] * inv_n;
     }
 #pragma unroll
     for (int q = 0; q < B; q++)
-        if (threadIdx.x + q * nthr < n) x[threadIdx.x + q * nthr] = xv[q];
+        if (int(threadIdx.x) + q * nthr < n) x[threadIdx.x + q * nthr] = xv[q] - (singular ? mean : T(0));
 }
 
 // dot product accumulated in T (FP32 on the mixed path: the bottom solve only
@@ -626,75 +518,54 @@ __device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int it
 }
 
 template <typename T>
-__device__ void bottom_solve(const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular) {
+__device__ void bottom_solve(const Level<T> &L, T ih2, T *x, const T *f, T *scr, int iters, int singular) {
     const int n = int(L.g.N);
-    const T ih2 = T(1) / T(L.g.h * L.g.h);
     if (n > BOT_REGS * CT) {
         cta_bicgstab(L, x, f, scr, iters, singular, ih2);
         return;
     }
-    if (n <= 32) {
-        if (threadIdx.x < 32) warp_bicgstab(L, x, f, scr, iters, singular, ih2);
-    } else {
-        // the fewest warps that hold the cells: their barriers cost less
-        const int per = (n + CT - 1) / CT, nthr = ((n + per - 1) / per + 31) & ~31;
-        if (int(threadIdx.x) < nthr) {
-            if (per == 1) team_bicgstab<T, 1>(L, x, f, scr, iters, singular, ih2, nthr);
-            else if (per == 2) team_bicgstab<T, 2>(L, x, f, scr, iters, singular, ih2, nthr);
-            else team_bicgstab<T, 3>(L, x, f, scr, iters, singular, ih2, nthr);
-        }
+    // the fewest warps that hold the cells: their barriers cost less
+    const int per = (n + CT - 1) / CT, nthr = ((n + per - 1) / per + 31) & ~31;
+    if (int(threadIdx.x) < nthr) {
+        if (per == 1) team_bicgstab<T, 1>(L, x, f, scr, iters, singular, ih2, nthr);
+        else team_bicgstab<T, BOT_REGS>(L, x, f, scr, iters, singular, ih2, nthr);
     }
     __syncthreads();
 }
 
-template <typename T>
+template <typename T, int SLMAX>
 __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &A, int rank) {
-    constexpr int CPT = CoarseCpt<T>::value;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    for (int q = threadIdx.x; q < A.roff; q += CT) sm[q] = T(0);
+    constexpr int B = sizeof(T);
+    for (int q = threadIdx.x * B; q < A.roff; q += CT * B) sm_at<T>(q) = T(0);
     __syncthreads();
-    {  // right-hand side of the first level from global memory
-        const CoarseLevel<T> &C = A.lev[0];
-        const Slab s = slab_of(C, rank);
-        const int nxy = int(C.L.g.nxy);
-        const T *f = C.L.f + (long long)s.k0 * nxy;
-        if (C.dist || rank == 0)
-            for (int q = threadIdx.x; q < nxy * s.np; q += CT) sm[C.foff + q] = f[q];
-    }
-    level_sync(A.nc > 1);
+    const int first = rank * A.lev[0].pp, nxy0 = int(A.lev[0].L.g.nxy);  // this CTA's planes of the first level
+    const int own0 = (A.lev[0].dist || rank == 0) ? nxy0 * max(0, min(A.lev[0].pp, A.lev[0].L.g.n[2] - first)) : 0;
+    for (int q = threadIdx.x; q < own0; q += CT) sm_at<T>(A.lev[0].foff + q * B) = A.lev[0].L.f[first * nxy0 + q];
+    if (A.nc > 1) cluster_sync();
+    else __syncthreads();
     const int nb = A.nl - 1;
-    Cells<T, CPT> R;
-    for (int l = 0; l < nb; l++) {
-        const CoarseLevel<T> &C = A.lev[l];
-        if (!C.dist && rank != 0) break;
-        const Slab s = slab_of(C, rank);
-        load_cells(C, s, R);
-        sweeps(sm, C, s, R, A.nu1);
-        restrict_down(sm, A, C, A.lev[l + 1], s, R);
+#pragma unroll 1
+    for (int step = 0; step <= 2 * nb; step++) {  // down, bottom, up
+        if (step == nb) {
+            const CoarseLevel<T> &C = A.lev[nb];
+            if (rank == 0)
+                bottom_solve(C.L, C.ih2, &sm_at<T>(C.eoff + int(C.L.g.nxy) * B), &sm_at<T>(C.foff), &sm_at<T>(A.roff),
+                             A.bot_iters, A.singular);
+            continue;
+        }
+        const bool up = step > nb;
+        const int l = up ? 2 * nb - step : step, dist = A.lev[l].dist;
+        if (!dist && rank != 0) continue;
+        // a spread level above ones of CTA 0 alone: every CTA waits for CTA 0
+        if (up && dist && !A.lev[l + 1].dist) cluster_sync();
+        const int own = int(A.lev[l].L.g.nxy) * A.lev[l].pp;
+        if (own <= CT) visit<T, 1>(A, l, rank, up);
+        else visit<T, SLMAX>(A, l, rank, up);
+        if (dist) cluster_sync();
+        else __syncthreads();
     }
-    if (rank == 0) {
-        const CoarseLevel<T> &C = A.lev[nb];
-        bottom_solve(C.L, sm + C.eoff + C.L.g.nxy, sm + C.foff, sm + A.roff, A.bot_iters, A.singular);
-    }
-    bool dist_below = false;  // the level below was spread: the cluster is in step already
-    for (int l = nb - 1; l >= 0; l--) {
-        const CoarseLevel<T> &C = A.lev[l];
-        if (!C.dist && rank != 0) continue;
-        const Slab s = slab_of(C, rank);
-        load_cells(C, s, R);
-        if (C.dist && !dist_below) cluster_sync();
-        dist_below = C.dist;
-        prolong_up(sm, C, A.lev[l + 1], s, R);
-        sweeps(sm, C, s, R, A.nu2);
-    }
-    const CoarseLevel<T> &C = A.lev[0];
-    if (C.dist || rank == 0) {
-        const Slab s = slab_of(C, rank);
-        const int nxy = int(C.L.g.nxy);
-        T *e = C.L.e + (long long)s.k0 * nxy;
-        for (int q = threadIdx.x; q < nxy * s.np; q += CT) e[q] = sm[C.eoff + nxy + q];
-    }
+    for (int q = threadIdx.x; q < own0; q += CT)
+        A.lev[0].L.e[first * nxy0 + q] = sm_at<T>(A.lev[0].eoff + (nxy0 + q) * B);
     if (A.nc > 1) cluster_sync();  // no CTA leaves while another may still read its shared memory
 }
 
@@ -702,14 +573,19 @@ template <typename T>
 __global__ void __launch_bounds__(CT, 1) coarse_vcycle_kernel(const __grid_constant__ CoarseArgs<T> A) {
     pdl_trigger();
     pdl_wait();
-    coarse_body(A, int(blockIdx.x));
+    coarse_body<T, CELLS_CLUSTER>(A, int(blockIdx.x));
 }
 
 // batched: one CTA per box (boxes already converged return at once)
 __global__ void __launch_bounds__(CT, 1) coarse_vcycle_batch_kernel(const CoarseArgs<float> *args,
                                                                     const SolveState *st) {
     if (st[blockIdx.x].done) return;
-    coarse_body(args[blockIdx.x], 0);
+    __shared__ CoarseArgs<float> A;
+    static_assert(sizeof(A) % sizeof(int) == 0, "copied by words");
+    for (int q = threadIdx.x; q < int(sizeof(A) / sizeof(int)); q += CT)
+        reinterpret_cast<int *>(&A)[q] = reinterpret_cast<const int *>(args + blockIdx.x)[q];
+    __syncthreads();
+    coarse_body<float, CELLS_ALONE>(A, 0);
 }
 
 // CTAs of a cluster on this device: 16 need as many free SMs in one GPC and the
@@ -743,8 +619,8 @@ static bool plan_coarse(CoarseArgs<T> &A, const Level<T> *levs, int nl, int nc) 
     if (nl < 1 || nl > COARSE_MAX_LEVELS) return false;
     std::memset(&A, 0, sizeof(A));
     A.nl = nl;
-    const int cap = CT * CoarseCpt<T>::value;
-    long long off = 4, scratch = 0;  // element 0 stays 0
+    const int cap = CT * (nc > 1 ? CELLS_CLUSTER : CELLS_ALONE), B = sizeof(T);
+    long long off = 16, scratch = 0;  // bytes; the element at 0 stays 0
     int used = 1;
     bool above_dist = true;
     for (int l = 0; l < nl; l++) {
@@ -752,13 +628,16 @@ static bool plan_coarse(CoarseArgs<T> &A, const Level<T> *levs, int nl, int nc) 
         CoarseLevel<T> &C = A.lev[l];
         if (g.N > 65535) return false;
         C.L = levs[l];
-        C.d0 = fast_div(g.n[0]);
-        C.d1 = fast_div(g.n[1]);
-        C.dh = fast_div(g.n[0] > 1 ? g.n[0] / 2 : 1);
         C.dist = nc > 1 && l + 1 < nl && above_dist && g.N > dist_min<T>();
         above_dist = C.dist;
         C.pp = C.dist ? 2 * ((g.n[2] + 2 * nc - 1) / (2 * nc)) : g.n[2];
         if (C.dist) used = std::max(used, (g.n[2] + C.pp - 1) / C.pp);
+        C.d0 = fast_div(g.n[0]);
+        C.d1 = fast_div(g.n[1]);
+        C.dh = fast_div(g.n[0] > 1 ? g.n[0] / 2 : 1);
+        C.dp = fast_div(C.pp);
+        C.h2 = T(g.h * g.h);
+        C.ih2 = T(1.0 / (g.h * g.h));
         const long long own = g.nxy * C.pp;
         if (l + 1 < nl) {
             if (own > cap) return false;
@@ -768,16 +647,18 @@ static bool plan_coarse(CoarseArgs<T> &A, const Level<T> *levs, int nl, int nc) 
             scratch = std::max(scratch, g.N > BOT_REGS * CT ? 6 * g.N : 2 * (g.N + 1));
         }
         C.eoff = int(off);
-        off += own + 2 * g.nxy;
-        C.foff = int(off);
-        off += own;
-        if (off > 65535) return false;  // neighbour indices are 16 bits
+        off += (own + 2 * g.nxy) * B;
+        if (off > 65535) return false;  // neighbour offsets are 16 bits
+    }
+    for (int l = 0; l < nl; l++) {
+        A.lev[l].foff = int(off);
+        off += levs[l].g.nxy * A.lev[l].pp * B;
     }
     for (A.nc = 1; A.nc < used;) A.nc *= 2;
     A.roff = int(off);
-    if ((off + scratch) * (long long)sizeof(T) > COARSE_MAX_SMEM) return false;
-    A.total = int(off + scratch);
-    return true;
+    off += scratch * B;
+    A.total = int(off);
+    return off <= COARSE_MAX_SMEM;
 }
 
 template <typename T>
@@ -797,7 +678,7 @@ void k_coarse_vcycle(cudaStream_t s, const Level<T> *levs, int nl, int nu1, int 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(A.nc);
     cfg.blockDim = dim3(CT);
-    cfg.dynamicSmemBytes = A.total * sizeof(T);
+    cfg.dynamicSmemBytes = A.total;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -840,7 +721,7 @@ size_t coarse_fill_args(void *dst, const Level<float> *levs, int nl, int nu1, in
     A.bot_iters = bot_iters;
     A.singular = singular;
     std::memcpy(dst, &A, sizeof(A));
-    return A.total * sizeof(float);
+    return A.total;
 }
 
 void k_coarse_vcycle_batch(cudaStream_t s, const void *dev_args, const SolveState *st, int nbox, size_t smem) {

@@ -31,8 +31,17 @@ struct DGeom {
 
 __host__ __device__ inline bool gper(const DGeom &g, int d) { return g.lo[d] == MX_BC_PERIODIC; }
 
+// FP64 levels keep the reciprocal of each cell's coefficient sum (the FP64
+// division takes eleven FMAs' time); FP32 divides as it goes.
 template <typename T>
-struct Level {
+struct LevelInverse {};
+template <>
+struct LevelInverse<double> {
+    double *di = nullptr;
+};
+
+template <typename T>
+struct Level : LevelInverse<T> {
     DGeom g;
     T *bx, *by, *bz;  // lo-face coefficients, one per cell
     T *hx, *hy, *hz;  // high-boundary face coefficients (non-periodic axes)
@@ -221,6 +230,8 @@ void k_finalize_max(cudaStream_t s, const double *partials, int nb, double *dst)
 // generic multigrid pieces (templated on the V-cycle precision)
 template <typename T>
 void k_coarsen_coeffs(cudaStream_t s, const Level<T> &fine, const Level<T> &coarse);
+// L.di = reciprocals of the cells' coefficient sums (FP64 levels)
+void k_inverse_diag(cudaStream_t s, const Level<double> &L);
 void k_round_coeffs(cudaStream_t s, const Level<double> &src, const Level<float> &dst);
 template <typename T>
 void k_residual64(cudaStream_t s, const Level<double> &L64, const double *phi, const double *f, T *rhat,

@@ -42,6 +42,23 @@ void k_coarsen_coeffs(cudaStream_t s, const Level<T> &fine, const Level<T> &coar
     coarsen_coeffs_kernel<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(fine, coarse);
 }
 
+// The FP64 smoother's divisions, once per solve: 23 FP64 operations per update
+// with the division inside, 8 with the stored reciprocal (the FP64 pipe bounds the
+// colour pass).
+__global__ void inverse_diag_kernel(Level<double> L) {
+    const DGeom &g = L.g;
+    const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (c >= g.N) return;
+    const int q = int(c), i = q % g.n[0], r = q / g.n[0], j = r % g.n[1], k = r / g.n[1];
+    double b[6];
+    face_coefs(L, i, j, k, c, b);
+    L.di[c] = gs_inverse(b);
+}
+
+void k_inverse_diag(cudaStream_t s, const Level<double> &L) {
+    inverse_diag_kernel<<<unsigned((L.g.N + 255) / 256), 256, 0, s>>>(L);
+}
+
 __global__ void round_coeffs_kernel(const double *a, float *b, long long n) {
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
         b[q] = float(a[q]);
@@ -205,7 +222,8 @@ __device__ __forceinline__ void rbgs_body(const Level<T> &L, int colour, T h2, i
         } else {
             nb_vals(g, L.e, i, j, k, c, v);
         }
-        L.e[c] = gs_update(b, v, L.f[c], h2);
+        if constexpr (sizeof(T) == sizeof(double)) L.e[c] = gs_update(b, v, L.f[c], h2, L.di[c]);
+        else L.e[c] = gs_update(b, v, L.f[c], h2);
     }
 }
 

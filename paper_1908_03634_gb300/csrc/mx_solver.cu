@@ -50,7 +50,10 @@ static void carve_level(Bump &b, Level<T> &L, const DGeom &g, bool coefs, bool f
 template <typename T>
 static void carve_hier(Bump &b, Hier<T> &H, const DGeom *gs, int nl, bool level0_coefs) {
     H.nlev = nl;
-    for (int l = 0; l < nl; l++) carve_level(b, H.lev[l], gs[l], l > 0 || level0_coefs, true);
+    for (int l = 0; l < nl; l++) {
+        carve_level(b, H.lev[l], gs[l], l > 0 || level0_coefs, true);
+        if constexpr (sizeof(T) == sizeof(double)) H.lev[l].di = b.take<T>(gs[l].N);
+    }
     H.bot_scratch = b.take<T>(7 * (size_t)gs[nl - 1].N);
 }
 
@@ -280,6 +283,8 @@ template void vcycle<double>(cudaStream_t, Hier<double> &, int, int, int, int, m
 template <typename T>
 static void build_hierarchy(cudaStream_t s, Hier<T> &H) {
     for (int l = 0; l + 1 < H.nlev; l++) k_coarsen_coeffs(s, H.lev[l], H.lev[l + 1]);
+    if constexpr (sizeof(T) == sizeof(double))
+        for (int l = 0; l < H.nlev; l++) k_inverse_diag(s, H.lev[l]);
 }
 
 // One refinement iteration after the residual: V-cycle, update, next residual.
