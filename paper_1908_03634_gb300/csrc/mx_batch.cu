@@ -146,11 +146,11 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
         for (int b = 0; b < nbox; b++)
             if (l < B->lc[b])
                 add_grid(work, b, zcf ? resid_restrict_fine_grid(B->box[b]->H32.lev[l].g, zcf)
-                                      : stencil_grid(B->box[b]->H32.lev[l + 1].g));
+                                      : stencil_grid_zc(B->box[b]->H32.lev[l + 1].g, ZC));
         B->rr[l].n = int(work.size()) - B->rr[l].off;
         B->pr[l].off = int(work.size());
         for (int b = 0; b < nbox; b++)
-            if (l < B->lc[b]) add_grid(work, b, stencil_grid(B->box[b]->H32.lev[l].g));
+            if (l < B->lc[b]) add_grid(work, b, stencil_grid_zc(B->box[b]->H32.lev[l].g, ZC));
         B->pr[l].n = int(work.size()) - B->pr[l].off;
     }
     B->df.off = int(work.size());

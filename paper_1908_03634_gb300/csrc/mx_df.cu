@@ -52,10 +52,10 @@ __global__ void mac_coeffs_df_kernel(Level<float> L, DFArrays D, FaceQ Q, const 
     const DGeom &g = L.g;
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int i = blockIdx.x * SX + tx, j = blockIdx.y * SY + ty;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const long long nxy = g.nxy;
-    const int k1 = min(k0 + ZC, nz);
+    const int k1 = min(k0 + zc, nz);
     const bool act = i < nx && j < ny;
     const bool wq = Q.x != nullptr;
     const dfloat zero = {0.f, 0.f};
@@ -267,10 +267,10 @@ __global__ void __launch_bounds__(SX *SY, 5) mac_rhs_df_kernel(DGeom g, const do
                                   const float *__restrict__ b0l, const double *__restrict__ sbar,
                                   float *__restrict__ fh, float *__restrict__ fl, double *part, dfloat hih) {
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     dfloat mx = {0.f, 0.f}, s1 = {0.f, 0.f};
     float s2 = 0.f;
-    df_div_block(g, ux, uy, uz, b0h, b0l, sbar, i, j, k0, min(k0 + ZC, g.n[2]), hih, [&](long long c, dfloat v) {
+    df_div_block(g, ux, uy, uz, b0h, b0l, sbar, i, j, k0, min(k0 + zc, g.n[2]), hih, [&](long long c, dfloat v) {
             fh[c] = v.h;
             fl[c] = v.l;
             df_absmax(mx, v);
@@ -286,10 +286,10 @@ __global__ void __launch_bounds__(SX *SY, 5) mac_divcheck_df_kernel(DGeom g, con
                                        const float *__restrict__ b0l, const double *__restrict__ sbar,
                                        const SolveState *st, double *part, dfloat hih) {
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     const dfloat cm = df_split(st->mean);
     dfloat mx = {0.f, 0.f};
-    df_div_block(g, ux, uy, uz, b0h, b0l, sbar, i, j, k0, min(k0 + ZC, g.n[2]), hih,
+    df_div_block(g, ux, uy, uz, b0h, b0l, sbar, i, j, k0, min(k0 + zc, g.n[2]), hih,
                  [&](long long, dfloat v) { df_absmax(mx, df_sub(v, cm)); });
     df_partials(mx, 0.f, dfloat{0.f, 0.f}, part + 3 * flat_bid());
 }

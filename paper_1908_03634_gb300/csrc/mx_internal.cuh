@@ -86,7 +86,14 @@ __device__ __forceinline__ void set_scale(SolveState *st, double sc) {
 // Maxima that propagate NaN.  fmax/fmaxf return the other operand when one is
 // NaN, so a norm built from them would report a finite value for a residual
 // holding NaN; every norm and its block and grid reductions use these instead.
-__device__ __forceinline__ double nmax(double a, double b) { return (a > b || a != a) ? a : b; }
+// The double form is for magnitudes (a, b >= 0 or NaN): their bit patterns order
+// like the values, with NaN on top, and integer comparisons leave the FP64 pipe
+// to the arithmetic (an FP64 comparison costs as much as an FP64 addition).
+__device__ __forceinline__ double nmax(double a, double b) {
+    const long long ia = __double_as_longlong(a) & 0x7fffffffffffffffll;
+    const long long ib = __double_as_longlong(b) & 0x7fffffffffffffffll;
+    return __longlong_as_double(ia > ib ? ia : ib);
+}
 __device__ __forceinline__ float nmaxf(float a, float b) {
     float r;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));

@@ -46,10 +46,10 @@ __global__ void mac_coeffs_kernel(Level<double> L, FaceQ Q, const double *__rest
                                   const double *__restrict__ beta0, double ih2x) {
     const DGeom &g = L.g;
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     if (i >= g.n[0] || j >= g.n[1]) return;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int k1 = min(k0 + ZC, nz);
+    const int k1 = min(k0 + zc, nz);
     const bool wq = Q.x != nullptr;
     for (int k = k0; k < k1; k++) {
         const long long c = i + (long long)nx * (j + (long long)ny * k);
@@ -155,10 +155,10 @@ __global__ void mac_rhs_kernel(DGeom g, const double *__restrict__ ux, const dou
                                const double *__restrict__ uz, const double *__restrict__ beta0,
                                const double *__restrict__ sbar, double *__restrict__ f, double *part, double hih) {
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     double mx = 0.0, s2 = 0.0, s1 = 0.0;
     if (i < g.n[0] && j < g.n[1])
-        div_column(g, ux, uy, uz, beta0, sbar, i, j, k0, min(k0 + ZC, g.n[2]), hih, [&](long long c, double v) {
+        div_column(g, ux, uy, uz, beta0, sbar, i, j, k0, min(k0 + zc, g.n[2]), hih, [&](long long c, double v) {
             f[c] = v;
             mx = nmax(mx, fabs(v));
             s2 = fma(v, v, s2);
@@ -205,7 +205,7 @@ __global__ void finalize_rhs_kernel(const double *part, int nb, SolveState *st, 
 
 void k_finalize_rhs(cudaStream_t s, const double *partials, int nb, SolveState *st, long long N, int remove_mean,
                     int stage) {
-    finalize_rhs_kernel<<<1, 1024, 0, s>>>(partials, nb, st, N, remove_mean, stage);
+    finalize_rhs_kernel<<<1, reduce_threads(nb), 0, s>>>(partials, nb, st, N, remove_mean, stage);
 }
 
 __global__ void sub_mean_norm_kernel(double *f, long long n, const SolveState *st, double *part) {
@@ -247,10 +247,10 @@ __device__ __forceinline__ void correct_face(const DGeom &g, int d, int p, long 
 __global__ void mac_correct_kernel(DGeom g, FaceQ Q, const double *__restrict__ phi, double *__restrict__ ux,
                                    double *__restrict__ uy, double *__restrict__ uz) {
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     if (i >= g.n[0] || j >= g.n[1]) return;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int k1 = min(k0 + ZC, nz);
+    const int k1 = min(k0 + zc, nz);
     for (int k = k0; k < k1; k++) {
         const long long c = i + (long long)nx * (j + (long long)ny * k);
         // x faces i (and nx on the last cell)
@@ -282,11 +282,11 @@ __global__ void mac_divcheck_kernel(DGeom g, const double *__restrict__ ux, cons
                                     const double *__restrict__ uz, const double *__restrict__ beta0,
                                     const double *__restrict__ sbar, const SolveState *st, double *part, double hih) {
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     const double cm = st->mean;
     double mx = 0.0, s2 = 0.0, s1 = 0.0;
     if (i < g.n[0] && j < g.n[1])
-        div_column(g, ux, uy, uz, beta0, sbar, i, j, k0, min(k0 + ZC, g.n[2]), hih,
+        div_column(g, ux, uy, uz, beta0, sbar, i, j, k0, min(k0 + zc, g.n[2]), hih,
                    [&](long long, double v) { mx = nmax(mx, fabs(v - cm)); });
     block_red3(mx, s2, s1);
     if (flat_tid() == 0) {
@@ -310,5 +310,5 @@ __global__ void finalize_max_kernel(const double *part, int nb, double *dst) {
 }
 
 void k_finalize_max(cudaStream_t s, const double *partials, int nb, double *dst) {
-    finalize_max_kernel<<<1, 1024, 0, s>>>(partials, nb, dst);
+    finalize_max_kernel<<<1, reduce_threads(nb), 0, s>>>(partials, nb, dst);
 }

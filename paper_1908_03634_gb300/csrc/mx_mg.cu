@@ -85,11 +85,11 @@ __global__ void residual64_kernel(Level<double> L, const double *__restrict__ ph
                                   T *__restrict__ rhat, const SolveState *st, double *part, double ih2) {
     const DGeom &g = L.g;
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     const double inv = st->inv_scale;
     double mx = 0.0, s2 = 0.0, s1 = 0.0;
     if (i < g.n[0] && j < g.n[1]) {
-        const int k1 = min(k0 + ZC, g.n[2]);
+        const int k1 = min(k0 + zc, g.n[2]);
         for (int k = k0; k < k1; k++) {
             const long long c = i + (long long)g.n[0] * (j + (long long)g.n[1] * k);
             double b[6], v[6];
@@ -163,7 +163,7 @@ __global__ void finalize_residual_kernel(const double *part, int nb, SolveState 
 }
 
 void k_finalize_residual(cudaStream_t s, const double *partials, int nb, SolveState *st, int scaled) {
-    launch_pdl(finalize_residual_kernel, dim3(1), dim3(1024), 0, s, partials, nb, st, scaled);
+    launch_pdl(finalize_residual_kernel, dim3(1), dim3(reduce_threads(nb)), 0, s, partials, nb, st, scaled);
 }
 
 // one block per box: partials [off[b], off[b] + cnt[b]) of r / scale; boxes
@@ -462,9 +462,9 @@ template <typename T>
 __global__ void apply_kernel(Level<T> L, const T *__restrict__ x, T *__restrict__ y, T ih2) {
     const DGeom &g = L.g;
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     if (i >= g.n[0] || j >= g.n[1]) return;
-    const int k1 = min(k0 + ZC, g.n[2]);
+    const int k1 = min(k0 + zc, g.n[2]);
     for (int k = k0; k < k1; k++) {
         const long long c = i + (long long)g.n[0] * (j + (long long)g.n[1] * k);
         T b[6], v[6];
@@ -641,7 +641,7 @@ __global__ void finalize_sum_kernel(const double *part, int nb, double *dst, dou
 }
 
 void k_finalize_sum(cudaStream_t s, const double *partials, int nb, double *dst, double scale) {
-    finalize_sum_kernel<<<1, 1024, 0, s>>>(partials, nb, dst, scale);
+    finalize_sum_kernel<<<1, reduce_threads(nb), 0, s>>>(partials, nb, dst, scale);
 }
 
 __global__ void sub_scalar_kernel(double *x, long long n, const double *val) {
@@ -659,10 +659,10 @@ __global__ void residual_plain_kernel(Level<double> L, const double *__restrict_
                                       double *__restrict__ r, double *part, double ih2) {
     const DGeom &g = L.g;
     const int i = blockIdx.x * SX + threadIdx.x, j = blockIdx.y * SY + threadIdx.y;
-    const int k0 = blockIdx.z * ZC;
+    const int zc = setup_zc(g), k0 = blockIdx.z * zc;
     double mx = 0.0, s2 = 0.0, s1 = 0.0;
     if (i < g.n[0] && j < g.n[1]) {
-        const int k1 = min(k0 + ZC, g.n[2]);
+        const int k1 = min(k0 + zc, g.n[2]);
         for (int k = k0; k < k1; k++) {
             const long long c = i + (long long)g.n[0] * (j + (long long)g.n[1] * k);
             double b[6], v[6];

@@ -100,7 +100,7 @@ extern "C" mx_status mx_residual_noalloc(const mx_geom *geom, const double *rho,
     if (!geom || !rho || !beta0 || !phi || !f || !r) return MX_ERR_ARG;
     if (check_geom(nullptr, geom, false) != MX_OK) return MX_ERR_ARG;
     const DGeom g = make_dgeom(geom);
-    const dim3 grid = stencil_grid(g);
+    const dim3 grid = stencil_grid_zc(g, ZC);
     const long long nb = (long long)grid.x * grid.y * grid.z;
     // more tiles than the fixed scratch holds, or a grid beyond the launch limits
     if (nb > NA_MAX_TILES || grid.y > 65535 || grid.z > 65535) return MX_ERR_ARG;

@@ -2126,7 +2126,7 @@ extern "C" mx_status mx_nodal_project(mx_ctx *c, const mx_geom *geom, double *ux
     } else
         nd_rhs_col_kernel<<<nd_node_grid(g), dim3(32, 8), 0, s>>>(g, ux, uy, uz, beta0, sbar, P->f64, c->partials, 0,
                                                                  c->state, 0.25 / g.h);
-    nd_finalize_rhs_kernel<<<1, 1024, 0, s>>>(c->partials, nd_node_blocks(g), c->state, o.remove_mean, 0);
+    nd_finalize_rhs_kernel<<<1, reduce_threads(nd_node_blocks(g)), 0, s>>>(c->partials, nd_node_blocks(g), c->state, o.remove_mean, 0);
     if (!o.remove_mean) {
         MX_CUDA(c, cudaMemcpyAsync(c->hstate, c->state, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
         MX_CUDA(c, cudaStreamSynchronize(s));
@@ -2143,7 +2143,7 @@ extern "C" mx_status mx_nodal_project(mx_ctx *c, const mx_geom *geom, double *ux
                                                   c->partials);
     else
         nd_rhs_final_kernel<<<nb, 256, 0, s>>>(g, P->f64, c->state, nullptr, nullptr, c->partials);
-    nd_finalize_rhs_kernel<<<1, 1024, 0, s>>>(c->partials, nb, c->state, 0, 1);
+    nd_finalize_rhs_kernel<<<1, reduce_threads(nb), 0, s>>>(c->partials, nb, c->state, 0, 1);
     if (mixed) {
         if (o.use_initial_guess) nd_split_kernel<<<nb, 256, 0, s>>>(phi, P->D.ph, P->D.pl, g.M);
         // else phi = 0 is set by the first residual's pass
@@ -2238,7 +2238,7 @@ extern "C" mx_status mx_nodal_project(mx_ctx *c, const mx_geom *geom, double *ux
     } else {
         nd_wsum_kernel<<<nb, 256, 0, s>>>(g, phi, c->partials);
     }
-    nd_wmean_finalize_kernel<<<1, 1024, 0, s>>>(c->partials, nb, &c->state->aux);
+    nd_wmean_finalize_kernel<<<1, reduce_threads(nb), 0, s>>>(c->partials, nb, &c->state->aux);
     k_sub_scalar(s, g.M, phi, &c->state->aux);
     if (mixed)
         nd_correct_df_kernel<<<cgrid, dim3(32, 8), 0, s>>>(g, rho, P->D, c->state, ux, uy, uz, df_host(0.25 / g.h),

@@ -162,9 +162,17 @@ __device__ __forceinline__ void reduce_partials3(const double *p, int nb, double
 // Launch shape of the cell-centred stencil kernels: (32 x 8) threads per block,
 // each thread walking ZC cells in z.
 constexpr int SX = 32, SY = 8, ZC = 8;
-inline dim3 stencil_grid(const DGeom &g) {
-    return dim3((g.n[0] + SX - 1) / SX, (g.n[1] + SY - 1) / SY, (g.n[2] + ZC - 1) / ZC);
+// Planes per block of the once-per-solve kernels and the FP64 residuals: ZC, and
+// halved while the grid has fewer than four blocks per SM.  Small boxes are
+// bound by the latency of a block's chain of planes: at 32^3 the FP64 residual
+// took 26 us on 16 blocks of 8 planes; computed alike by host and kernels.
+__host__ __device__ inline int setup_zc(const DGeom &g) {
+    const int bxy = ((g.n[0] + SX - 1) / SX) * ((g.n[1] + SY - 1) / SY);
+    int sh = 3;
+    while (sh > 0 && (long long)bxy * ((g.n[2] + (1 << sh) - 1) >> sh) < 4 * 152) sh--;
+    return 1 << sh;
 }
+static_assert(ZC == 8, "setup_zc starts from ZC");
 // z-chunk for a level with bxy blocks per chunk of planes: `cap` planes per
 // thread (8 unless tuned) on large levels, fewer (down to 1) until the grid
 // has >= 16 blocks per SM, so small levels are not latency-bound on a few
@@ -180,7 +188,10 @@ inline dim3 stencil_grid_zc(const DGeom &g, int zc) {
 inline int stencil_zc(const DGeom &g, int cap = ZC) {
     return zchunk((long long)((g.n[0] + SX - 1) / SX) * ((g.n[1] + SY - 1) / SY), g.n[2], cap);
 }
+inline dim3 stencil_grid(const DGeom &g) { return stencil_grid_zc(g, setup_zc(g)); }
 inline int stencil_blocks(const DGeom &g) {
     dim3 d = stencil_grid(g);
     return int(d.x * d.y * d.z);
 }
+// threads of a one-block reduction of nb partials (its FP64 sums cost by the warp)
+inline int reduce_threads(int nb) { return nb >= 1024 ? 1024 : (nb + 31) / 32 * 32; }
