@@ -25,6 +25,7 @@
 #include "mx_coarse.cuh"
 #include "mx_rbgs.cuh"
 #include "mx_stencil.cuh"
+#include "mx_team.cuh"
 
 constexpr int CT = 1024;         // threads per CTA
 constexpr int BOT_REGS = 2;      // bottom solves of up to BOT_REGS * CT cells keep their vectors in registers
@@ -264,9 +265,6 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
     }
 }
 
-// The bottom solve's scalar divisions: they set its step lengths, so the fast
-// forms (a subroutine's instructions would cost more than its arithmetic).
-__device__ __forceinline__ float sdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b); }
 
 // BiCGStab on L x = f (x starts at 0), projected onto mean-free vectors when
@@ -287,7 +285,6 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
                                               T ih2, int nthr) {
     __shared__ T red[2][4][32];
     const int n = int(L.g.N), nx = L.g.n[0], ny = L.g.n[1], nz = L.g.n[2], nxy = nx * ny;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nthr >> 5;
     T b[B][6], den[B], xv[B], r[B], r0[B], p[B], v[B];
     unsigned nb[B][3];
     if (threadIdx.x < 2) scr[threadIdx.x * (n + 1) + n] = T(0);
@@ -315,40 +312,11 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
         }
         den[q] = radd(radd(radd(b[q][0], b[q][1]), radd(b[q][2], b[q][3])), radd(b[q][4], b[q][5]));
     }
-    auto barrier = [&] { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); };
-    // Sums of a[0..4) over the team, the same bits in every thread.  The four sums
-    // share the shuffles (each exchange halves what a lane still carries: 6 in
-    // place of 20), lane group g = lane / 8 ends with sum g.  The two buffers
-    // alternate: a barrier lies between a reduction's reads and the writes of the
-    // next but one.
-    int turn = 0;
-    auto group_sum = [&](T k) {
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-        return k;
-    };
-    auto team_sum = [&]() {
-        const bool up16 = lane & 16, up8 = lane & 8;
-        T k0 = up16 ? a[2] : a[0], k1 = up16 ? a[3] : a[1];
-        k0 += __shfl_xor_sync(0xffffffffu, up16 ? a[0] : a[2], 16);
-        k1 += __shfl_xor_sync(0xffffffffu, up16 ? a[1] : a[3], 16);
-        T k = (up8 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up8 ? k0 : k1, 8);
-        k = group_sum(k);
-        if (nw > 1) {
-            if ((lane & 7) == 0) red[turn][lane >> 3][warp] = k;
-            barrier();
-            k = T(0);
-            for (int q = lane & 7; q < nw; q += 8) k += red[turn][lane >> 3][q];
-            k = group_sum(k);
-            turn ^= 1;
-        }
-#pragma unroll
-        for (int m = 0; m < 4; m++) a[m] = __shfl_sync(0xffffffffu, k, 8 * m);
-    };
+    TeamSum<T> team(red, nthr);
     const T inv_n = T(1) / T(n);
     T mean = T(0), rho1 = T(0), rho = T(1), alpha = T(1), omega = T(1), tol2 = T(0);
     // step -1: the mean of f and ||f - mean||^2; then the iterations
-    team_sum();
+    team.sum(a);
     if (singular) mean = a[0] * inv_n;
     a[0] = a[1] = a[2] = a[3] = T(0);
 #pragma unroll
@@ -357,7 +325,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
         r0[q] = r[q];
         a[0] = rfma(r[q], r[q], a[0]);
     }
-    team_sum();
+    team.sum(a);
     rho1 = a[0];
     if (rho1 > T(0)) {
         tol2 = rho1 * T(1e-8);  // 1e-4 relative: ample for a multigrid bottom solve
@@ -375,7 +343,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
 #pragma unroll
                 for (int q = 0; q < B; q++)
                     if (int(threadIdx.x) + q * nthr < n) e[threadIdx.x + q * nthr] = w[q];
-                barrier();
+                team.barrier();
                 a[0] = a[1] = a[2] = a[3] = T(0);
 #pragma unroll
                 for (int q = 0; q < B; q++) {
@@ -388,7 +356,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
                     a[2] = rfma(y[q], y[q], a[2]);
                     a[3] = rfma(y[q], w[q], a[3]);
                 }
-                team_sum();
+                team.sum(a);
                 if (h == 0) {
                     stop = a[0] == T(0);
                     if (stop) break;
@@ -417,7 +385,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
     if (singular) {
 #pragma unroll
         for (int q = 0; q < B; q++) a[0] += xv[q];
-        team_sum();
+        team.sum(a);
         mean = a[0] * inv_n;
     }
 #pragma unroll

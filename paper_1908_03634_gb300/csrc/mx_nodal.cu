@@ -21,6 +21,7 @@
 #include "mx_dfmath.cuh"
 #include "mx_solver.cuh"
 #include "mx_stencil.cuh"
+#include "mx_team.cuh"
 
 struct NGeom {
     int n[3];   // cells
@@ -524,7 +525,7 @@ __global__ void nd_apply_kernel(NLevel<T> L, const T *x, T *y) {
 // BiCGStab on the coarsest nodal level (one CTA).  The nodal operator is
 // symmetric in the w-weighted inner product; singular problems (no Dirichlet
 // nodes) are projected onto weighted-mean-free vectors.
-constexpr int NBT = 256;
+constexpr int NBT = 512;
 
 template <typename T>
 __device__ T nd_wdot(const NGeom &g, const T *a, const T *b, int weighted) {
@@ -562,12 +563,127 @@ __device__ void nd_wmean0(const NGeom &g, T *x) {
     __syncthreads();
 }
 
+// The same solve for at most NBT nodes, one per thread: couplings and vectors in
+// registers, the vector the operator is applied to in shared memory (element n
+// holds 0), the two applications of an iteration through one rolled body with one
+// reduction each (the sums' recurrences as in the cell-centred bottom solve).
+// The cost is instruction fetch and the latency of the sums: 240 nodes took 318 us
+// per V-cycle when every product re-read the 8 cells and every sum was its own
+// block-wide reduction.
+template <typename T>
+__device__ __forceinline__ void nd_team_bicgstab(const NLevel<T> &L, int iters, int nthr) {
+    __shared__ T vec[2][NBT + 1];
+    __shared__ float red[2][4][32];
+    const NGeom &g = L.g;
+    const int n = int(g.M), q = threadIdx.x;
+    TeamSum<float> team(red, nthr);
+    if (q < 2) vec[q][n] = T(0);
+    T coef[20], den = T(0), inv = T(0);
+    unsigned nb[10];
+    float w = 0.f;
+#pragma unroll
+    for (int m = 0; m < 20; m++) coef[m] = T(0);
+#pragma unroll
+    for (int m = 0; m < 10; m++) nb[m] = unsigned(n) | (unsigned(n) << 16);
+    T r = T(0);
+    if (q < n) {
+        int a, b, c, m = 0;
+        node_of(g, q, a, b, c);
+        T s[2][2][2];
+        cell_ring(g, L.sigma, a, b, c, s);
+        // the couplings in for_couplings' order, unrolled: they stay in registers
+#pragma unroll
+        for (int o = 0; o < 27; o++) {
+            const int ox = o % 3 - 1, oy = o / 3 % 3 - 1, oz = o / 9 - 1;
+            if ((ox != 0) + (oy != 0) + (oz != 0) < 2) continue;
+            T k = T(0);
+#pragma unroll
+            for (int d = 0; d < 8; d++) {
+                const int dx = d & 1, dy = (d >> 1) & 1, dz = d >> 2;
+                if ((ox == 0 || dx == (ox > 0)) && (oy == 0 || dy == (oy > 0)) && (oz == 0 || dz == (oz > 0)))
+                    k += s[dz][dy][dx];
+            }
+            const int na = node_wrap(g, 0, a + ox), nn = node_wrap(g, 1, b + oy), nc = node_wrap(g, 2, c + oz);
+            const unsigned t = (na >= 0 && nn >= 0 && nc >= 0) ? unsigned(nidx(g, na, nn, nc)) : unsigned(n);
+            coef[m] = k;
+            nb[m >> 1] = (m & 1) ? (nb[m >> 1] & 0xffffu) | (t << 16) : (nb[m >> 1] & 0xffff0000u) | t;
+            den += k;
+            m++;
+        }
+        w = node_w(g, a, b, c);
+        inv = T(1) / (T(12) * T(w) * T(g.h * g.h));
+        r = L.f[q];
+    }
+    float a[4] = {w * float(r), w, 0.f, 0.f};
+    team.sum(a);
+    const float wsum = a[1];
+    if (q < n) r -= T(a[0] / wsum);  // compatibility (all nodal problems here are singular)
+    const T r0 = r;
+    T x = T(0), p = T(0), v = T(0);
+    a[0] = w * float(r) * float(r);
+    a[1] = a[2] = a[3] = 0.f;
+    team.sum(a);
+    float rho1 = a[0], rho = 1.f, alpha = 1.f, omega = 1.f;
+    if (rho1 > 0.f) {
+        const float tol2 = rho1 * 1e-8f;
+#pragma unroll 1
+        for (int it = 0; it < iters; it++) {
+            if (rho1 == 0.f || omega == 0.f) break;
+            p = r + T(sdiv(rho1 * alpha, rho * omega)) * (p - T(omega) * v);
+            T u = p, y = T(0);
+            bool stop = false;
+#pragma unroll 1
+            for (int h = 0; h < 2; h++) {  // y = L u: v = L p, then t = L s
+                if (q < n) vec[h][q] = u;
+                team.barrier();
+                T n0 = T(0), n1 = T(0);
+#pragma unroll
+                for (int m = 0; m < 10; m++) {
+                    n0 += coef[2 * m] * vec[h][nb[m] & 0xffffu];
+                    n1 += coef[2 * m + 1] * vec[h][nb[m] >> 16];
+                }
+                y = ((n0 + n1) - den * u) * inv;
+                const float wy = w * float(y), fu = float(u), fy = float(y);
+                a[0] = wy * float(r0);
+                a[1] = w * fu * fu;
+                a[2] = wy * fy;
+                a[3] = wy * fu;
+                team.sum(a);
+                if (h == 0) {
+                    stop = a[0] == 0.f;
+                    if (stop) break;
+                    alpha = sdiv(rho1, a[0]);
+                    v = y;
+                    u = r - T(alpha) * y;
+                }
+            }
+            if (stop) break;
+            const bool small = a[1] <= tol2;
+            omega = !small && a[2] > 0.f ? sdiv(a[3], a[2]) : 0.f;
+            x += T(alpha) * p + T(omega) * u;
+            r = u - T(omega) * y;
+            if (small || a[1] - omega * (2.f * a[3] - omega * a[2]) <= tol2) break;
+            rho = rho1;
+            rho1 = -omega * a[0];
+        }
+    }
+    a[0] = w * float(x);
+    a[1] = a[2] = a[3] = 0.f;
+    team.sum(a);
+    if (q < n) L.e[q] = x - T(a[0] / wsum);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int iters) {
     pdl_trigger();
     pdl_wait();
     const NGeom &g = L.g;
     const int n = int(g.M);
+    if (n <= NBT) {
+        const int nthr = (n + 31) & ~31;
+        if (int(threadIdx.x) < nthr) nd_team_bicgstab(L, iters, nthr);
+        return;
+    }
     T *x = L.e, *r = scr, *r0 = scr + n, *p = scr + 2 * n, *v = scr + 3 * n, *sv = scr + 4 * n, *tv = scr + 5 * n;
     for (int q = threadIdx.x; q < n; q += NBT) r[q] = L.f[q];
     __syncthreads();

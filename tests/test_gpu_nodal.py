@@ -199,3 +199,22 @@ def test_smoother_option_rejected_where_not_offered(mx, ctx):
         with pytest.raises(mx.MXError) as e:
             mx.mx_nodal_project(ctx, g, *u, one, one, z, phi, mx.default_opts(smoother=bad))
         assert e.value.status == mx.MX_ERR_ARG
+
+
+@pytest.mark.parametrize("n,bc", [((2, 2, 2), (P, P, N)), ((4, 4, 4), (P, P, P)), ((6, 10, 14), (P, P, N)),
+                                  ((12, 20, 28), (N, N, N)), ((14, 14, 14), (N, N, N)), ((18, 14, 22), (N, N, N))])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_nodal_bottom_sizes(mx, ctx, n, bc, prec):
+    """The bottom solve on 12, 8, 120, 192, 512 (as many nodes as threads) and 960
+    nodes (vectors in memory): phi within the projection's 1e-8 of the oracle."""
+    g = geom(n, bc)
+    rng = np.random.default_rng(3)
+    cs = O.cell_shape(g)
+    rho, beta0 = np.exp(0.5 * rng.standard_normal(cs)), np.exp(0.5 * rng.standard_normal(cs))
+    u, sbar = [rng.standard_normal(cs) for _ in range(3)], rng.standard_normal(cs)
+    _, ref, info = O.nd_project(g, u, rho, beta0, sbar, tol=1e-13, maxit=400)
+    assert info["ok"]
+    phi = torch.zeros(O.node_shape(g), dtype=torch.float64, device=DEV)
+    mx.mx_nodal_project(ctx, g, *[cuda(t) for t in u], cuda(rho), cuda(beta0), cuda(sbar), phi,
+                        mx.default_opts(prec=prec))
+    assert np.abs(phi.cpu().numpy() - ref).max() <= 1e-8 * np.abs(ref).max()
