@@ -171,7 +171,11 @@ def roofline_per_vcycle(ncell, nu1, nu2, w, ms_solve, vcycles, hbm, loop_ms=None
     return out
 
 
-def launches_per_solve(g, o, vcycles, graph, krylov=0):
+SWEEP_CELLS = 6 << 20       # levels from here on run single-pass sweeps (mx_opts.fused = 0)
+CLUSTER_CELLS = 32768       # levels the coarse end takes, at most (a cube's)
+
+
+def launches_per_solve(g, o, vcycles, graph, krylov=0, sweep_cells=None, coarse_cells=4096):
     """Kernels the library launches for one mixed-precision MAC solve (fill
     included), from the solver's structure: setup 13 + first residual 2; per
     refinement iteration the V-cycle's launches on the levels above the coarse
@@ -180,16 +184,19 @@ def launches_per_solve(g, o, vcycles, graph, krylov=0):
     (+1 condition kernel inside the graph); finish 6 (4 without a mean to
     remove).  FCG (krylov = 1) adds 4 per iteration: the dot product, its
     finalize, the direction/stencil pass and the step finalize.  Checked against
-    the ncu launch lists of the planar 256^3 solve."""
+    the ncu launch lists of the planar 256^3 solve.  sweep_cells: levels of at
+    least so many cells run single-pass sweeps without o.fused; coarse_cells: the
+    largest level of the coarse end."""
     dims = [list(g.n)]
     while all(d % 2 == 0 and d >= 4 for d in dims[-1]):
         dims.append([d // 2 for d in dims[-1]])
     nlev = len(dims)
     ncell = [d[0] * d[1] * d[2] for d in dims]
-    ldown = next((l for l in range(nlev) if ncell[l] <= 4096), nlev - 1)
+    ldown = next((l for l in range(nlev) if ncell[l] <= coarse_cells), nlev - 1)
     per_iter = 1 + 2 + (1 if graph else 0) + (4 if krylov else 0)
     for l in range(ldown):
-        fused = o.fused and ncell[l] >= (1 << 18) and dims[l][0] % 2 == 0
+        least = (1 << 18) if o.fused else sweep_cells
+        fused = least and ncell[l] >= least and dims[l][0] % 4 == 0 and dims[l][0] >= 32
         per_iter += (o.nu1 + 1 + o.nu2) if fused else (2 * o.nu1 + 1 + 1 + 2 * o.nu2)
     setup = 1 + 1 + (nlev - 1) + 4 + 2
     singular = all(b != 2 for b in tuple(g.lo) + tuple(g.hi))  # no Dirichlet face
@@ -281,7 +288,7 @@ def run_mx(args):
     last = infos[-1]
     assert all(i["status"] == 0 for i in infos), infos[-1]
     vcycles = statistics.mean(i["vcycles"] for i in infos[Wm:])
-    launches = int(round(K * launches_per_solve(g, tuned, vcycles, graph, kry)))
+    launches = int(round(K * launches_per_solve(g, tuned, vcycles, graph, kry, SWEEP_CELLS, CLUSTER_CELLS)))
 
     # ---- plain FP64 solve (the comparison) ----
     fp64 = None
@@ -361,7 +368,7 @@ def run_mx(args):
     sm_ms, sm_n = trace["smooth_fine"]
     per_launch_ms = sm_ms / max(sm_n, 1)
     # the tuned smoother: two colour passes (12 B/cell each) or single-pass sweeps (24 B/cell)
-    fused0 = bool(tuned.fused) and ncell >= (1 << 18) and g.n[0] % 2 == 0
+    fused0 = ncell >= ((1 << 18) if tuned.fused else SWEEP_CELLS) and g.n[0] % 4 == 0
     sweep_bytes = 2 * bpc["smooth_fine"] if fused0 else bpc["smooth_fine"]
     achieved = sweep_bytes * ncell / (per_launch_ms * 1e-3) / 1e9
     r_ms, r_n = trace["resid64"]
@@ -374,7 +381,7 @@ def run_mx(args):
         pass
     if fused0:
         traffic = None  # the ncu figure is for the colour-pass kernel
-    roofline = {"kernel": ("rbgs_march_kernel (finest level, one red+black sweep)" if fused0 else
+    roofline = {"kernel": ("rbgs_sweep_kernel (finest level, one red+black sweep)" if fused0 else
                            "rbgs_kernel<float> (finest level, one colour)"), "bound": "hbm",
                 "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                 "peak_source": peak_src, "traffic": traffic,

@@ -86,8 +86,11 @@ typedef struct {
     int use_graph;         /* 1: run the refinement loop as one CUDA graph */
     int nu1, nu2;          /* pre/post smoothing sweeps (red+black each) */
     int bottom_iters;      /* BiCGStab iteration cap on the coarsest grid */
-    int fused;             /* 1: single-pass tile sweeps with the prolongation fused on load;
-                              0: two-pass colour kernels (default; bit-identical results) */
+    int fused;             /* FP32 smoothing of a level: single-pass sweeps with the prolongation
+                              fused on load, or two colour kernels (bit-identical results).
+                              0 (default): sweeps on levels that outgrow the L2 cache;
+                              1: on every level of 2^18 cells or more that allows them
+                              (n[0] a multiple of 4, at least 32) */
     int tile_z;            /* cells per thread along z in the stencil kernels' tiles (the
                               largest z-chunk; smaller levels use fewer): 0 = default
                               (8 MAC, 16 nodal), else 1, 2, 4, 8 or 16; results do not

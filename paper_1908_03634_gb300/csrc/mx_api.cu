@@ -7,6 +7,7 @@
 #include <memory>
 
 #include "mx_coarse.cuh"
+#include "mx_rbgs.cuh"
 #include "mx_stencil.cuh"
 #include "mx_solver.cuh"
 
@@ -146,7 +147,7 @@ mx_status mx_create(mx_ctx **out, int device, void *stream) {
         cudaMallocHost(&c->hstate, sizeof(SolveState) * 4) != cudaSuccess ||
         cudaMalloc(&c->partials, sizeof(double) * 3 * c->max_partials) != cudaSuccess ||
         cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess ||
-        coarse_init() != cudaSuccess) {
+        coarse_init() != cudaSuccess || rbgs_init() != cudaSuccess) {
         cudaGetLastError();
         mx_destroy(c);
         return MX_ERR_CUDA;

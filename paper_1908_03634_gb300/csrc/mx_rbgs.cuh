@@ -10,20 +10,21 @@ enum { RB_PLAIN = 0, RB_ZERO = 1, RB_PROLONG = 2 };
 // (two-pass colour passes, the single-pass sweep, the batched and coarse-end
 // kernels) evaluates the update with exactly these operations, so they agree
 // bit for bit whatever FMA contractions the compiler would choose in each.
-// The FP32 update divides with the reciprocal-based fast division (within 2 ulp
-// for denominators below 2^126, far above any face-coefficient sum here), whose
-// result is the product with the reciprocal of the denominator bit for bit: a
-// kernel that updates a cell many times keeps gs_inverse(b) (the same bits on
-// 5e8 random pairs with exponents within 2^+-63).  FP64 multiplies with a
-// reciprocal within 2 ulp.  The smoother only sets the V-cycle's contraction, the
-// refinement loop the accuracy.
+// FP32 multiplies with the hardware's approximate reciprocal of the diagonal (1
+// ulp; subnormal sums, far below any face-coefficient sum here, count as 0), FP64
+// with a reciprocal within 2 ulp.  The smoother only sets the V-cycle's
+// contraction, the refinement loop the accuracy.
 __device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float rinv(float a) { return __fdividef(1.f, a); }
+__device__ __forceinline__ float rinv(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
 __device__ __forceinline__ double rinv(double a) { return rcp64(a); }
 
 // 1 / sum_f b_f of a cell's row
@@ -49,12 +50,14 @@ __device__ __forceinline__ T gs_update(const T b[6], const T v[6], T f, T h2, T 
     return rmul(gs_numerator(b, v, f, h2), inv);
 }
 __device__ __forceinline__ float gs_update(const float b[6], const float v[6], float f, float h2) {
-    const float num = gs_numerator(b, v, f, h2);
-    return __fdividef(num, radd(radd(radd(b[0], b[1]), radd(b[2], b[3])), radd(b[4], b[5])));
+    return gs_update(b, v, f, h2, gs_inverse(b));
 }
 
 // Whether the single-pass sweep supports this level (n_x even, periodic extents >= 2).
 bool rbgs_fused_ok(const DGeom &g);
+
+// Allow the sweep kernels their shared memory (once per device, outside any capture).
+cudaError_t rbgs_init();
 
 // e_out = one red+black sweep applied to e_in (mode RB_ZERO: e_in = 0;
 // RB_PROLONG: e_in + piecewise-constant prolongation of coarse->e).

@@ -188,14 +188,21 @@ void destroy_plans(mx_ctx *c) {
 // V-cycle on the correction equation L e = r (level-0 f holds r, e is zeroed here)
 
 // V-cycle on the correction equation L e = r (level-0 f holds r).
-//  * levels of >= FUSED_MIN_CELLS cells (FP32, fused = 1): single-pass sweeps
+//  * FP32 levels of >= SWEEP_MIN_CELLS cells (with fused = 1, of >=
+//    FUSED_MIN_CELLS): single-pass sweeps
 //    ping-ponging between e and e2; the first pre-sweep starts from e = 0
 //    without reading it and the first post-sweep applies the prolongation on
 //    load; the first output buffer is chosen so that the result ends in e;
 //  * other levels above the coarse end: two-pass colour kernels in place;
 //  * the coarse end (the levels that fit one cluster's shared memory, down to the
 //    bottom): one launch; without such a level, a BiCGStab bottom kernel.
+//
+// A sweep moves half the bytes of two colour passes but takes more of the SMs'
+// shared-memory pipe, so the line lies where e, f and the coefficients (20 B per
+// cell) outgrow the 126 MB L2: measured, 256^3 96 us a sweep against 112 us,
+// 160x192x224 42 against 46, and 128^3, out of L2, 21 against 18.
 constexpr long long FUSED_MIN_CELLS = 1LL << 18;
+constexpr long long SWEEP_MIN_CELLS = 6LL << 20;
 
 template <typename T>
 int coarse_start(const Hier<T> &H, int clustered) {
@@ -210,8 +217,8 @@ void vcycle(cudaStream_t s, Hier<T> &H, int nu1, int nu2, int bot_iters, int sin
     const int nl = H.nlev;
     const int lc = coarse_start(H, 1);
     const int ldown = lc < nl ? lc : nl - 1;  // levels with their own kernels
-    const bool can_fuse = sizeof(T) == sizeof(float) && fused && nu1 >= 1 && nu2 >= 1;
-    auto is_fused = [&](int l) { return can_fuse && H.lev[l].g.N >= FUSED_MIN_CELLS && rbgs_fused_ok(H.lev[l].g); };
+    const bool can_fuse = sizeof(T) == sizeof(float) && nu1 >= 1 && nu2 >= 1;
+    auto is_fused = [&](int l) { return can_fuse && H.lev[l].g.N >= (fused ? FUSED_MIN_CELLS : SWEEP_MIN_CELLS) && rbgs_fused_ok(H.lev[l].g); };
     T *cur[MX_MAXLEV];
     for (int l = 0; l < ldown; l++) {
         Level<T> &L = H.lev[l];

@@ -1,0 +1,53 @@
+"""The single-pass red-black sweep against the two colour passes at the edges of
+its tiles: widths of exactly one tile, one column of pairs into the next and not
+a multiple of four pairs; rows that fill the last tile, leave one row in it or
+wrap; chunks of one plane run and of several; walls, Dirichlet and periodic faces
+on every axis.  Both do per cell the same rounded operations, so after two
+V-cycles phi is equal bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1908_03634_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+P, N, D = W.PERIODIC, W.NEUMANN, W.DIRICHLET
+DEV = torch.device("cuda:0")
+
+
+@pytest.fixture(scope="module")
+def mx():
+    from paper_1908_03634_gb300 import build as b
+    b.build()
+    import paper_1908_03634_gb300 as m
+    return m
+
+
+@pytest.fixture(scope="module")
+def ctx(mx):
+    c = mx.mx_create(0)
+    yield c
+    mx.mx_destroy(c)
+
+
+@pytest.mark.parametrize("n,bc", [((60, 112, 48), (P, P, N)), ((64, 98, 48), (D, D, D)), ((36, 128, 64), (P, D, P)),
+                                  ((124, 30, 72), (D, P, D)), ((244, 16, 72), (N, N, P)), ((240, 140, 8), (P, N, D)),
+                                  ((32, 16, 512), (D, N, N)), ((512, 4, 128), (N, P, D))])
+@pytest.mark.parametrize("nu", [(1, 1), (2, 3)])
+def test_sweep_bits(mx, ctx, n, bc, nu):
+    g = W.Geom(n, 1.0 / n[0], bc, bc)
+    rng = np.random.default_rng(2)
+    cs = mx.cell_shape(g)
+    cuda = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    rho, beta0 = cuda(np.exp(0.5 * rng.standard_normal(cs))), cuda(np.exp(0.5 * rng.standard_normal(cs)))
+    sbar = cuda(rng.standard_normal(cs))
+    u = W._periodic_faces(g, [torch.from_numpy(rng.standard_normal(g.face_shape(d))) for d in range(3)])
+    out = []
+    for fused in (0, 1):
+        phi = torch.zeros(cs, dtype=torch.float64, device=DEV)
+        st, info = mx.mx_mac_project(ctx, g, *[cuda(t.numpy()) for t in u], rho, beta0, sbar, phi,
+                                     mx.default_opts(fused=fused, nu1=nu[0], nu2=nu[1], max_outer=2),
+                                     allow=(mx.MX_OK, mx.MX_ERR_NOCONV))
+        assert info["vcycles"] == 2 and np.isfinite(info["rel_resid"])
+        out.append(phi.cpu().numpy())
+    assert np.array_equal(out[0], out[1])
