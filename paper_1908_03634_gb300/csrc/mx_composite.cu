@@ -371,113 +371,244 @@ struct CompCoefs {
     const double *c[3], *f[3];
 };
 // r = f - L phi with the cached face coefficients (the operator of
-// comp_apply_*_kernel), and per-block maxima of |r| in part (if non-null)
-__global__ void comp_resid_coarse_kernel(CompGeom G, CompCoefs B, const double *__restrict__ pc,
-                                         const double *__restrict__ pf, const double *__restrict__ f,
-                                         double *__restrict__ out, double *part) {
-    const long long N = (long long)G.n[0] * G.n[1] * G.n[2];
+// comp_apply_*_kernel), and per-block maxima of |r| in part (if non-null).
+//
+// The FP64 pipe bounds these: 13 operations per cell with the factor 1/h^2 taken
+// once (the flux b (phi_nb - phi) of a face enters as one subtraction and one FMA).
+// The cells whose rows need more -- fine cells on the patch's boundary (ghost
+// values), coarse cells across it (the means of four fine fluxes) -- would hold up
+// whole warps of plain rows, so blocks past the first `nmain` take just them, listed
+// face by face; the others march columns in 32 x 8 tiles, RZ planes each.  128^3 +
+// 128^3: 113 and 144 us with every row in one loop over the cells.
+constexpr int RZ = 8;
+struct RTile {
+    int i, j, k0, k1;
+    bool in;
+};
+__host__ __device__ inline int resid_main_blocks(const int n[3]) {
+    return ((n[0] + 31) / 32) * ((n[1] + 7) / 8) * ((n[2] + RZ - 1) / RZ);
+}
+__device__ __forceinline__ RTile resid_tile(const int n[3]) {
+    const int bx = (n[0] + 31) / 32, by = (n[1] + 7) / 8, q = blockIdx.x, r = q / bx;
+    RTile t;
+    t.i = (q - r * bx) * 32 + int(threadIdx.x & 31);
+    t.j = (r % by) * 8 + int(threadIdx.x >> 5);
+    t.k0 = (r / by) * RZ;
+    t.k1 = min(t.k0 + RZ, n[2]);
+    t.in = t.i < n[0] && t.j < n[1];
+    return t;
+}
+__device__ __forceinline__ void block_max(double rmax, double *part) {
+    if (!part) return;
+    double z1 = 0.0, z2 = 0.0;
+    block_red3(rmax, z1, z2);
+    if (threadIdx.x == 0) part[3 * blockIdx.x] = rmax;
+}
+
+// coarse cells across the patch's faces, in the order x low, x high, y low, ...
+__host__ __device__ inline int coarse_shell(const CompGeom &G) {
+    const int a = G.phi[0] - G.plo[0], b = G.phi[1] - G.plo[1], c = G.phi[2] - G.plo[2];
+    return 2 * (b * c + a * c + a * b);
+}
+__device__ __forceinline__ void coarse_shell_cell(const CompGeom &G, int q, int c[3], int &d, int &s) {
+    for (d = 0; d < 3; d++) {
+        const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
+        const int l1 = G.phi[t1] - G.plo[t1], l2 = G.phi[t2] - G.plo[t2];
+        for (s = 1; s >= -1; s -= 2) {  // s: from the cell towards the patch
+            if (q < l1 * l2) {
+                c[d] = s > 0 ? G.plo[d] - 1 : G.phi[d];
+                c[t1] = G.plo[t1] + q % l1;
+                c[t2] = G.plo[t2] + q / l1;
+                return;
+            }
+            q -= l1 * l2;
+        }
+    }
+}
+// sum over the faces of coarse cell c of b (phi_nb - phi_c), the face towards the
+// patch (dp, sp) excepted
+__device__ __forceinline__ double coarse_row(const CompGeom &G, const CompCoefs &B, const double *__restrict__ pc,
+                                             const int c[3], double p0, int dp, int sp) {
+    double acc = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        int m[3] = {G.n[0], G.n[1], G.n[2]};
+        m[d] += 1;
+#pragma unroll
+        for (int s = -1; s <= 1; s += 2) {
+            if (d == dp && s == sp) continue;
+            int face[3] = {c[0], c[1], c[2]}, nb[3] = {c[0], c[1], c[2]};
+            if (s > 0) face[d] += 1;
+            nb[d] += s;
+            const bool beyond = nb[d] < 0 || nb[d] >= G.n[d];
+            if (beyond) nb[d] = nb[d] < 0 ? G.n[d] - 1 : 0;
+            // beyond a Dirichlet face (b = 2 beta0/rho) or a wall (b = 0): 0
+            const double v = beyond && G.lo[d] != MX_BC_PERIODIC ? 0.0 : pc[cix(G, nb[0], nb[1], nb[2])];
+            acc = fma(B.c[d][face_ix(m, face)], v - p0, acc);
+        }
+    }
+    return acc;
+}
+__global__ void __launch_bounds__(256) comp_resid_coarse_kernel(CompGeom G, CompCoefs B, const double *__restrict__ pc,
+                                                                const double *__restrict__ pf,
+                                                                const double *__restrict__ f, double *__restrict__ out,
+                                                                double *part, int nmain) {
     const double iH2 = 1.0 / (G.H * G.H), ihH = 1.0 / (G.h * G.H);
     double rmax = 0.0;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N; q += (long long)gridDim.x * blockDim.x) {
-        int c[3];
-        coarse_ijk(G, q, c);
-        if (in_patch(G, c)) {
-            out[q] = 0.0;
-            continue;
-        }
-        const double p0 = pc[q];
-        double acc = 0.0;
-        for (int d = 0; d < 3; d++) {
-            int m[3] = {G.n[0], G.n[1], G.n[2]};
-            m[d] += 1;
-            for (int s = -1; s <= 1; s += 2) {
-                int face[3] = {c[0], c[1], c[2]};
-                if (s > 0) face[d] += 1;
-                const double b = B.c[d][face_ix(m, face)];
-                int nb[3] = {c[0], c[1], c[2]};
-                nb[d] += s;
-                if (nb[d] < 0 || nb[d] >= G.n[d]) {
-                    if (G.lo[d] != MX_BC_PERIODIC) {
-                        acc -= b * p0 * iH2;  // Dirichlet (b = 2 beta0/rho) or wall (b = 0)
-                        continue;
-                    }
-                    nb[d] = (nb[d] + G.n[d]) % G.n[d];
+    if (int(blockIdx.x) < nmain) {
+        const RTile t = resid_tile(G.n);
+        if (t.in)
+            for (int k = t.k0; k < t.k1; k++) {
+                const int c[3] = {t.i, t.j, k};
+                const long long q = cix(G, t.i, t.j, k);
+                int within = 0, across = 0;  // axes on which c lies in the patch's range, or one cell off it
+                for (int d = 0; d < 3; d++) {
+                    within += c[d] >= G.plo[d] && c[d] < G.phi[d];
+                    across += c[d] == G.plo[d] - 1 || c[d] == G.phi[d];
                 }
-                if (!in_patch(G, nb)) {
-                    acc += b * (pc[cix(G, nb[0], nb[1], nb[2])] - p0) * iH2;
-                    continue;
+                if (within == 3) {
+                    out[q] = 0.0;
+                } else if (!(within == 2 && across == 1)) {
+                    const double r = fma(-iH2, coarse_row(G, B, pc, c, pc[q], -1, 0), f[q]);
+                    rmax = nmax(rmax, fabs(r));
+                    out[q] = r;
                 }
-                // coarse-fine face: the mean of the four fine fluxes
-                const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-                const int Fd = 2 * (nb[d] - G.plo[d]) + (s > 0 ? 0 : 1);
-                int mf[3] = {G.nf[0], G.nf[1], G.nf[2]};
-                mf[d] += 1;
-                double mm = 0.0;
-                for (int a = 0; a < 2; a++)
-                    for (int e = 0; e < 2; e++) {
-                        int F[3];
-                        F[d] = Fd;
-                        F[t1] = 2 * (c[t1] - G.plo[t1]) + a;
-                        F[t2] = 2 * (c[t2] - G.plo[t2]) + e;
-                        int ff[3] = {F[0], F[1], F[2]};
-                        if (s < 0) ff[d] += 1;  // the fine cell's high face
-                        int C[3];
-                        const double g = ghost(G, pc, pf, F, d, -s, C);
-                        mm += B.f[d][face_ix(mf, ff)] * (pf[fix_(G, F[0], F[1], F[2])] - g);
-                    }
-                acc += 0.25 * mm * ihH;
             }
+    } else {
+        const int q = (int(blockIdx.x) - nmain) * 256 + int(threadIdx.x);
+        if (q < coarse_shell(G)) {
+            int c[3], d, s;
+            coarse_shell_cell(G, q, c, d, s);
+            const long long qc = cix(G, c[0], c[1], c[2]);
+            double acc = coarse_row(G, B, pc, c, pc[qc], d, s) * iH2;
+            // the face towards the patch: the mean of the four fine fluxes
+            const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
+            int mf[3] = {G.nf[0], G.nf[1], G.nf[2]};
+            mf[d] += 1;
+            double mm = 0.0;
+            for (int e = 0; e < 4; e++) {
+                int F[3];
+                F[d] = s > 0 ? 0 : G.nf[d] - 1;
+                F[t1] = 2 * (c[t1] - G.plo[t1]) + (e >> 1);
+                F[t2] = 2 * (c[t2] - G.plo[t2]) + (e & 1);
+                int ff[3] = {F[0], F[1], F[2]};
+                if (s < 0) ff[d] += 1;  // the fine cell's high face
+                int C[3];
+                const double g = ghost(G, pc, pf, F, d, -s, C);
+                mm = fma(B.f[d][face_ix(mf, ff)], pf[fix_(G, F[0], F[1], F[2])] - g, mm);
+            }
+            acc = fma(0.25 * ihH, mm, acc);
+            const double r = f[qc] - acc;
+            rmax = fabs(r);
+            out[qc] = r;
         }
-        acc = f[q] - acc;
-        rmax = nmax(rmax, fabs(acc));
-        out[q] = acc;
     }
-    if (part) {
-        double z1 = 0.0, z2 = 0.0;
-        block_red3(rmax, z1, z2);
-        if (threadIdx.x == 0) part[3 * blockIdx.x] = rmax;
-    }
+    block_max(rmax, part);
 }
-__global__ void comp_resid_fine_kernel(CompGeom G, CompCoefs B, const double *__restrict__ pc,
-                                       const double *__restrict__ pf, const double *__restrict__ f,
-                                       double *__restrict__ out, double *part) {
-    const long long N = (long long)G.nf[0] * G.nf[1] * G.nf[2];
+
+// fine cells on the patch's boundary: the planes k = 0 and last, then the rows
+// j = 0 and last of the others, then their first and last cells
+__host__ __device__ inline int fine_shell(const CompGeom &G) {
+    return G.nf[0] * G.nf[1] * G.nf[2] - (G.nf[0] - 2) * (G.nf[1] - 2) * (G.nf[2] - 2);
+}
+__device__ __forceinline__ void fine_shell_cell(const CompGeom &G, int q, int F[3]) {
+    const int nx = G.nf[0], ny = G.nf[1], nz = G.nf[2];
+    if (q < 2 * nx * ny) {
+        F[2] = q < nx * ny ? 0 : nz - 1;
+        const int r = q < nx * ny ? q : q - nx * ny;
+        F[1] = r / nx;
+        F[0] = r - F[1] * nx;
+        return;
+    }
+    q -= 2 * nx * ny;
+    if (q < 2 * nx * (nz - 2)) {
+        const int r = q / nx;
+        F[0] = q - r * nx;
+        F[1] = r & 1 ? ny - 1 : 0;
+        F[2] = 1 + (r >> 1);
+        return;
+    }
+    q -= 2 * nx * (nz - 2);
+    const int r = q >> 1;
+    F[0] = q & 1 ? nx - 1 : 0;
+    F[2] = 1 + r / (ny - 2);
+    F[1] = 1 + r % (ny - 2);
+}
+__global__ void __launch_bounds__(256) comp_resid_fine_kernel(CompGeom G, CompCoefs B, const double *__restrict__ pc,
+                                                              const double *__restrict__ pf,
+                                                              const double *__restrict__ f, double *__restrict__ out,
+                                                              double *part, int nmain) {
     const double ih2 = 1.0 / (G.h * G.h);
+    const int nx = G.nf[0], ny = G.nf[1], nz = G.nf[2];
     double rmax = 0.0;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N; q += (long long)gridDim.x * blockDim.x) {
-        int F[3];
-        fine_ijk(G, q, F);
-        const double p0 = pf[q];
-        double acc = 0.0;
-        for (int d = 0; d < 3; d++) {
-            int m[3] = {G.nf[0], G.nf[1], G.nf[2]};
-            m[d] += 1;
-            for (int s = -1; s <= 1; s += 2) {
-                int face[3] = {F[0], F[1], F[2]};
-                if (s > 0) face[d] += 1;
-                const double b = B.f[d][face_ix(m, face)];
-                int nb[3] = {F[0], F[1], F[2]};
-                nb[d] += s;
-                if (nb[d] >= 0 && nb[d] < G.nf[d]) {
-                    acc += b * (pf[fix_(G, nb[0], nb[1], nb[2])] - p0) * ih2;
-                } else {
-                    int C[3];
-                    acc += b * (ghost(G, pc, pf, F, d, s, C) - p0) * ih2;
-                }
+    if (int(blockIdx.x) < nmain) {
+        const RTile t = resid_tile(G.nf);
+        if (t.in && t.i > 0 && t.i < nx - 1 && t.j > 0 && t.j < ny - 1) {
+            const int k0 = max(t.k0, 1), k1 = min(t.k1, nz - 1);
+            const long long xy = (long long)nx * ny;
+            long long q = fix_(G, t.i, t.j, k0);
+            const double *__restrict__ bx = B.f[0] + t.i + (long long)(nx + 1) * (t.j + (long long)ny * k0);
+            const double *__restrict__ by = B.f[1] + t.i + (long long)nx * (t.j + (long long)(ny + 1) * k0);
+            const double *__restrict__ bz = B.f[2] + q;  // z faces: low face of cell k at plane k
+            double p0 = k0 < k1 ? pf[q] : 0.0, pd = k0 < k1 ? pf[q - xy] : 0.0;
+            for (int k = k0; k < k1; k++, q += xy, bx += (long long)(nx + 1) * ny, by += (long long)nx * (ny + 1), bz += xy) {
+                const double pu = pf[q + xy];
+                double acc = bx[0] * (pf[q - 1] - p0);
+                acc = fma(bx[1], pf[q + 1] - p0, acc);
+                acc = fma(by[0], pf[q - nx] - p0, acc);
+                acc = fma(by[nx], pf[q + nx] - p0, acc);
+                acc = fma(bz[0], pd - p0, acc);
+                acc = fma(bz[xy], pu - p0, acc);
+                const double r = fma(-ih2, acc, f[q]);
+                rmax = nmax(rmax, fabs(r));
+                out[q] = r;
+                pd = p0;
+                p0 = pu;
             }
         }
-        acc = f[q] - acc;
-        rmax = nmax(rmax, fabs(acc));
-        out[q] = acc;
+    } else {
+        const int q = (int(blockIdx.x) - nmain) * 256 + int(threadIdx.x);
+        if (q < fine_shell(G)) {
+            int F[3];
+            fine_shell_cell(G, q, F);
+            const long long qf = fix_(G, F[0], F[1], F[2]);
+            const double p0 = pf[qf];
+            double acc = 0.0;
+            for (int d = 0; d < 3; d++) {
+                int m[3] = {nx, ny, nz};
+                m[d] += 1;
+                for (int s = -1; s <= 1; s += 2) {
+                    int face[3] = {F[0], F[1], F[2]}, nb[3] = {F[0], F[1], F[2]}, C[3];
+                    if (s > 0) face[d] += 1;
+                    nb[d] += s;
+                    const double v = nb[d] >= 0 && nb[d] < G.nf[d] ? pf[fix_(G, nb[0], nb[1], nb[2])]
+                                                                   : ghost(G, pc, pf, F, d, s, C);
+                    acc = fma(B.f[d][face_ix(m, face)], v - p0, acc);
+                }
+            }
+            const double r = fma(-ih2, acc, f[qf]);
+            rmax = fabs(r);
+            out[qf] = r;
+        }
     }
-    if (part) {
-        double z1 = 0.0, z2 = 0.0;
-        block_red3(rmax, z1, z2);
-        if (threadIdx.x == 0) part[3 * blockIdx.x] = rmax;
-    }
+    block_max(rmax, part);
 }
 
-
+// the two residuals; part (if non-null) takes resid_parts(G) partial maxima, the
+// coarse level's first
+int resid_coarse_blocks(const CompGeom &G) { return resid_main_blocks(G.n) + (coarse_shell(G) + 255) / 256; }
+int resid_fine_blocks(const CompGeom &G) { return resid_main_blocks(G.nf) + (fine_shell(G) + 255) / 256; }
+int resid_parts(const CompGeom &G) { return resid_coarse_blocks(G) + resid_fine_blocks(G); }
+void k_resid_coarse(cudaStream_t s, const CompGeom &G, const CompCoefs &B, const double *pc, const double *pf,
+                    const double *f, double *out, double *part) {
+    comp_resid_coarse_kernel<<<resid_coarse_blocks(G), 256, 0, s>>>(G, B, pc, pf, f, out, part, resid_main_blocks(G.n));
+}
+void k_resid_fine(cudaStream_t s, const CompGeom &G, const CompCoefs &B, const double *pc, const double *pf,
+                  const double *f, double *out, double *part) {
+    comp_resid_fine_kernel<<<resid_fine_blocks(G), 256, 0, s>>>(G, B, pc, pf, f, out,
+                                                                part ? part + 3 * resid_coarse_blocks(G) : nullptr,
+                                                                resid_main_blocks(G.nf));
+}
 
 // f = D(beta0 U) - beta0 Sbar on the uncovered coarse cells (0 on covered ones)
 // and the fine cells, in place over the divergence; partials (max |f|,
@@ -1009,13 +1140,13 @@ void comp_body(cudaStream_t s, mx_ctx *c, CompPlan &P, double *phi_c, double *ph
     comp_coarse_rhs_kernel<<<nbc, 256, 0, s>>>(G, P.rcb, P.rfb, dst, HC.lev[0].f);
     vcycle(s, HC, o.nu1, o.nu2, o.bottom_iters, P.singular, nullptr, 0, zcap);
     comp_coarse_update_kernel<<<nb, 256, 0, s>>>(G, phi_c, phi_f, HC.lev[0].e, dst, nbc);
-    comp_resid_fine_kernel<<<nbf, 256, 0, s>>>(G, P.B, phi_c, phi_f, P.ff, P.rfb, nullptr);
+    k_resid_fine(s, G, P.B, phi_c, phi_f, P.ff, P.rfb, nullptr);
     comp_fine_rhs_kernel<<<nbf, 256, 0, s>>>(Nf, P.rfb, dst, HF.lev[0].f);
     vcycle(s, HF, o.nu1, o.nu2, o.bottom_iters, 0, nullptr, 0, zcap);
     comp_fine_update_kernel<<<nbf, 256, 0, s>>>(Nf, phi_f, HF.lev[0].e, dst);
-    comp_resid_coarse_kernel<<<nbc, 256, 0, s>>>(G, P.B, phi_c, phi_f, P.fc, P.rcb, part);
-    comp_resid_fine_kernel<<<nbf, 256, 0, s>>>(G, P.B, phi_c, phi_f, P.ff, P.rfb, part + 3 * nbc);
-    comp_decide_kernel<<<1, 1024, 0, s>>>(part, nb, dst);
+    k_resid_coarse(s, G, P.B, phi_c, phi_f, P.fc, P.rcb, part);
+    k_resid_fine(s, G, P.B, phi_c, phi_f, P.ff, P.rfb, part);
+    comp_decide_kernel<<<1, 1024, 0, s>>>(part, resid_parts(G), dst);
 }
 }  // namespace
 
@@ -1046,7 +1177,7 @@ extern "C" mx_status mx_mac_project_composite(mx_ctx *c, const mx_geom *geom, co
     cudaStream_t s = c->stream;
     const long long Nc = (long long)G.n[0] * G.n[1] * G.n[2], Nf = (long long)G.nf[0] * G.nf[1] * G.nf[2];
     const int nbc = gs_blocks(Nc), nbf = gs_blocks(Nf), nb = nbc + nbf;
-    if ((st = ensure_partials(c, nb))) return st;
+    if ((st = ensure_partials(c, std::max(nb, resid_parts(G))))) return st;
     CompPlan *Pp = get_comp_plan(c, G, geom, &st);
     if (!Pp) return st;
     CompPlan &P = *Pp;
@@ -1101,9 +1232,9 @@ extern "C" mx_status mx_mac_project_composite(mx_ctx *c, const mx_geom *geom, co
     }
 
     // first residual, then the refinement loop (a conditional graph, or from the host)
-    comp_resid_coarse_kernel<<<nbc, 256, 0, s>>>(G, P.B, phi_c, phi_f, P.fc, P.rcb, part);
-    comp_resid_fine_kernel<<<nbf, 256, 0, s>>>(G, P.B, phi_c, phi_f, P.ff, P.rfb, part + 3 * nbc);
-    comp_decide_kernel<<<1, 1024, 0, s>>>(part, nb, dst);
+    k_resid_coarse(s, G, P.B, phi_c, phi_f, P.fc, P.rcb, part);
+    k_resid_fine(s, G, P.B, phi_c, phi_f, P.ff, P.rfb, part);
+    comp_decide_kernel<<<1, 1024, 0, s>>>(part, resid_parts(G), dst);
     MX_CUDA(c, cudaMemcpyAsync(c->hstate, dst, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
     MX_CUDA(c, cudaStreamSynchronize(s));
     if (!c->hstate->done) {
