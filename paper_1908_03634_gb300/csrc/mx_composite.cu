@@ -1041,10 +1041,11 @@ struct CompPlan {
     MacPlan *pc = nullptr, *pf = nullptr;
     void *mem = nullptr;
     double *fc, *rcb, *rm, *bm, *ff, *rfb;
+    double *pcb, *pfb;  // phi of the refinement loop (the caller's arrays change from call to call)
     CompCoefs B;
     // the refinement loop's graph and what it was captured with
     cudaGraphExec_t graph = nullptr;
-    const void *k_pc = nullptr, *k_pf = nullptr, *k_part = nullptr;
+    const void *k_part = nullptr;
     int k_nu1 = -1, k_nu2 = -1, k_bot = -1, k_zcap = -1;
     ~CompPlan() {
         if (graph) cudaGraphExecDestroy(graph);
@@ -1090,7 +1091,7 @@ CompPlan *get_comp_plan(mx_ctx *c, const CompGeom &G, const mx_geom *geom, mx_st
         return nullptr;
     }
     const long long Nc = gc.N, Nf = gf.N;
-    long long nface_c[3], nface_f[3], tot = 4 * Nc + 2 * Nf;
+    long long nface_c[3], nface_f[3], tot = 5 * Nc + 3 * Nf;
     for (int d = 0; d < 3; d++) {
         nface_c[d] = (Nc / G.n[d]) * (G.n[d] + 1);
         nface_f[d] = (Nf / G.nf[d]) * (G.nf[d] + 1);
@@ -1110,7 +1111,9 @@ CompPlan *get_comp_plan(mx_ctx *c, const CompGeom &G, const mx_geom *geom, mx_st
     P->bm = x + 3 * Nc;
     P->ff = x + 4 * Nc;
     P->rfb = P->ff + Nf;
-    x = P->rfb + Nf;
+    P->pcb = P->rfb + Nf;
+    P->pfb = P->pcb + Nc;
+    x = P->pfb + Nf;
     double *bcoef[6];
     for (int d = 0; d < 3; d++) {
         bcoef[d] = x;
@@ -1227,28 +1230,28 @@ extern "C" mx_status mx_mac_project_composite(mx_ctx *c, const mx_geom *geom, co
     }
     comp_scale_kernel<<<1, 1, 0, s>>>(dst);
     if (!o.use_initial_guess) {
-        MX_CUDA(c, cudaMemsetAsync(phi_c, 0, sizeof(double) * Nc, s));
-        MX_CUDA(c, cudaMemsetAsync(phi_f, 0, sizeof(double) * Nf, s));
+        MX_CUDA(c, cudaMemsetAsync(P.pcb, 0, sizeof(double) * Nc, s));
+        MX_CUDA(c, cudaMemsetAsync(P.pfb, 0, sizeof(double) * Nf, s));
+    } else {
+        MX_CUDA(c, cudaMemcpyAsync(P.pcb, phi_c, sizeof(double) * Nc, cudaMemcpyDeviceToDevice, s));
+        MX_CUDA(c, cudaMemcpyAsync(P.pfb, phi_f, sizeof(double) * Nf, cudaMemcpyDeviceToDevice, s));
     }
 
     // first residual, then the refinement loop (a conditional graph, or from the host)
-    k_resid_coarse(s, G, P.B, phi_c, phi_f, P.fc, P.rcb, part);
-    k_resid_fine(s, G, P.B, phi_c, phi_f, P.ff, P.rfb, part);
+    k_resid_coarse(s, G, P.B, P.pcb, P.pfb, P.fc, P.rcb, part);
+    k_resid_fine(s, G, P.B, P.pcb, P.pfb, P.ff, P.rfb, part);
     comp_decide_kernel<<<1, 1024, 0, s>>>(part, resid_parts(G), dst);
     MX_CUDA(c, cudaMemcpyAsync(c->hstate, dst, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
     MX_CUDA(c, cudaStreamSynchronize(s));
     if (!c->hstate->done) {
         if (o.use_graph) {
-            if (!P.graph || P.k_pc != phi_c || P.k_pf != phi_f || P.k_part != part || P.k_nu1 != o.nu1 ||
-                P.k_nu2 != o.nu2 || P.k_bot != o.bottom_iters || P.k_zcap != zcap) {
+            if (!P.graph || P.k_part != part || P.k_nu1 != o.nu1 || P.k_nu2 != o.nu2 || P.k_bot != o.bottom_iters || P.k_zcap != zcap) {
                 if (P.graph) {
                     cudaGraphExecDestroy(P.graph);
                     P.graph = nullptr;
                 }
-                st = capture_while_graph(c, &P.graph, [&](cudaStream_t cs) { comp_body(cs, c, P, phi_c, phi_f, o, zcap); });
+                st = capture_while_graph(c, &P.graph, [&](cudaStream_t cs) { comp_body(cs, c, P, P.pcb, P.pfb, o, zcap); });
                 if (st) return st;
-                P.k_pc = phi_c;
-                P.k_pf = phi_f;
                 P.k_part = part;
                 P.k_nu1 = o.nu1;
                 P.k_nu2 = o.nu2;
@@ -1258,13 +1261,16 @@ extern "C" mx_status mx_mac_project_composite(mx_ctx *c, const mx_geom *geom, co
             MX_CUDA(c, cudaGraphLaunch(P.graph, s));
         } else {
             for (;;) {
-                comp_body(s, c, P, phi_c, phi_f, o, zcap);
+                comp_body(s, c, P, P.pcb, P.pfb, o, zcap);
                 MX_CUDA(c, cudaMemcpyAsync(c->hstate, dst, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
                 MX_CUDA(c, cudaStreamSynchronize(s));
                 if (c->hstate->done) break;
             }
         }
     }
+
+    MX_CUDA(c, cudaMemcpyAsync(phi_c, P.pcb, sizeof(double) * Nc, cudaMemcpyDeviceToDevice, s));
+    MX_CUDA(c, cudaMemcpyAsync(phi_f, P.pfb, sizeof(double) * Nf, cudaMemcpyDeviceToDevice, s));
 
     // normalisation (zero volume-weighted mean of the unknowns when singular), the
     // covered coarse phi, the velocity correction on both levels, the check

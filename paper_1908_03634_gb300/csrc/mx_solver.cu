@@ -405,9 +405,7 @@ mx_status capture_while_graph(mx_ctx *c, cudaGraphExec_t *exec, const std::funct
 template <typename T>
 static mx_status run_loop_graph(mx_ctx *c, MacPlan &P, Hier<T> &H, double *phi, const mx_opts &o, int singular, int nb) {
     cudaStream_t s = c->stream;
-    // the FP64 loop updates phi in place; the mixed loop never touches it
-    const void *kphi = sizeof(T) == sizeof(double) ? (const void *)phi : nullptr;
-    if (!P.graph || P.graph_phi != kphi || P.graph_nu1 != o.nu1 || P.graph_nu2 != o.nu2 ||
+    if (!P.graph || P.graph_nu1 != o.nu1 || P.graph_nu2 != o.nu2 ||
         P.graph_bot != o.bottom_iters || P.graph_fused != o.fused || P.graph_tilez != o.tile_z ||
         P.graph_krylov != o.krylov) {
         if (P.graph) {
@@ -417,7 +415,6 @@ static mx_status run_loop_graph(mx_ctx *c, MacPlan &P, Hier<T> &H, double *phi, 
         mx_status st = capture_while_graph(
             c, &P.graph, [&](cudaStream_t cs) { ir_step(cs, c, P, H, phi, o, singular, nb, nullptr); });
         if (st) return st;
-        P.graph_phi = kphi;
         P.graph_nu1 = o.nu1;
         P.graph_nu2 = o.nu2;
         P.graph_bot = o.bottom_iters;
@@ -558,14 +555,18 @@ extern "C" mx_status mx_mac_project(mx_ctx *c, const mx_geom *geom, double *ux, 
         }
     } else {
         k_sub_mean_norm(s, g, f64, c->state, c->partials, nbr);
-        if (!o.use_initial_guess) MX_CUDA(c, cudaMemsetAsync(phi, 0, sizeof(double) * g.N, s));
+        // the loop's phi is the plan's: its graph then holds for every caller's array
+        if (!o.use_initial_guess) MX_CUDA(c, cudaMemsetAsync(P->L64.e, 0, sizeof(double) * g.N, s));
+        else MX_CUDA(c, cudaMemcpyAsync(P->L64.e, phi, sizeof(double) * g.N, cudaMemcpyDeviceToDevice, s));
     }
     k_finalize_rhs(s, c->partials, nbr, c->state, g.N, 0, 1);
     prof_end(c, s, MX_PH_SETUP, 0);
 
     if (o.prec == MX_PREC_MIXED) st = run_ir<float>(c, *P, P->H32, phi, o, singular);
-    else st = run_ir<double>(c, *P, P->H64, phi, o, singular);
+    else st = run_ir<double>(c, *P, P->H64, P->L64.e, o, singular);
     if (st) return st;
+    if (o.prec != MX_PREC_MIXED)
+        MX_CUDA(c, cudaMemcpyAsync(phi, P->L64.e, sizeof(double) * g.N, cudaMemcpyDeviceToDevice, s));
     prof_begin(c, s, MX_PH_FINISH);
     // mixed: phi from its double-float form, with the partial sums of phi
     if (o.prec == MX_PREC_MIXED) k_df_final(s, g.N, P->D, c->state, phi, singular ? c->partials : nullptr);
