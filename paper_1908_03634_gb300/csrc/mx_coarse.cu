@@ -28,6 +28,7 @@
 #include "mx_team.cuh"
 
 constexpr int CT = 1024;         // threads per CTA
+constexpr int BOT_ONE = 256;      // ... of up to BOT_ONE cells hold one cell per thread
 constexpr int BOT_REGS = 2;      // bottom solves of up to BOT_REGS * CT cells keep their vectors in registers
 constexpr int COARSE_NC = 16;    // CTAs of the cluster (8 where the device cannot place 16)
 
@@ -268,7 +269,10 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
 __device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b); }
 
 // BiCGStab on L x = f (x starts at 0), projected onto mean-free vectors when
-// the problem is singular; stops at relative residual 1e-4 or `iters`.  Each of
+// the problem is singular; stops at relative residual 1e-4 or `iters`.  The
+// operator is preconditioned from the right with its diagonal (v = L D^-1 p, so
+// the residuals are those of L x = f): the stratified coefficients vary a hundredfold
+// over the bottom level.  Each of
 // nthr threads (whole warps) holds up to B cells (cell t + q nthr): coefficients
 // and vectors stay in registers, and the vector the operator is applied to passes
 // through shared memory (element n holds 0 for faces without a neighbour).
@@ -285,7 +289,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
                                               T ih2, int nthr) {
     __shared__ T red[2][4][32];
     const int n = int(L.g.N), nx = L.g.n[0], ny = L.g.n[1], nz = L.g.n[2], nxy = nx * ny;
-    T b[B][6], den[B], xv[B], r[B], r0[B], p[B], v[B];
+    T b[B][6], den[B], dinv[B], xv[B], r[B], r0[B], p[B], v[B];
     unsigned nb[B][3];
     if (threadIdx.x < 2) scr[threadIdx.x * (n + 1) + n] = T(0);
     T a[4] = {T(0), T(0), T(0), T(0)};
@@ -311,6 +315,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
             a[0] += r[q];
         }
         den[q] = radd(radd(radd(b[q][0], b[q][1]), radd(b[q][2], b[q][3])), radd(b[q][4], b[q][5]));
+        dinv[q] = den[q] != T(0) ? rinv(den[q]) : T(0);
     }
     TeamSum<T> team(red, nthr);
     const T inv_n = T(1) / T(n);
@@ -342,7 +347,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
                 T *e = scr + h * (n + 1);
 #pragma unroll
                 for (int q = 0; q < B; q++)
-                    if (int(threadIdx.x) + q * nthr < n) e[threadIdx.x + q * nthr] = w[q];
+                    if (int(threadIdx.x) + q * nthr < n) e[threadIdx.x + q * nthr] = rmul(w[q], dinv[q]);
                 team.barrier();
                 a[0] = a[1] = a[2] = a[3] = T(0);
 #pragma unroll
@@ -350,7 +355,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
                     const T s0 = rfma(b[q][0], e[nb[q][0] & 0xffffu], rmul(b[q][1], e[nb[q][0] >> 16]));
                     const T s1 = rfma(b[q][2], e[nb[q][1] & 0xffffu], rmul(b[q][3], e[nb[q][1] >> 16]));
                     const T s2 = rfma(b[q][4], e[nb[q][2] & 0xffffu], rmul(b[q][5], e[nb[q][2] >> 16]));
-                    y[q] = rmul(rfma(-den[q], w[q], radd(radd(s0, s1), s2)), ih2);
+                    y[q] = rmul(rfma(-den[q], rmul(w[q], dinv[q]), radd(radd(s0, s1), s2)), ih2);
                     a[0] = rfma(r0[q], y[q], a[0]);
                     a[1] = rfma(w[q], w[q], a[1]);
                     a[2] = rfma(y[q], y[q], a[2]);
@@ -373,7 +378,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
             omega = !small && a[2] > T(0) ? sdiv(a[3], a[2]) : T(0);
 #pragma unroll
             for (int q = 0; q < B; q++) {
-                xv[q] = rfma(omega, w[q], rfma(alpha, p[q], xv[q]));
+                xv[q] = rfma(rfma(omega, w[q], rmul(alpha, p[q])), dinv[q], xv[q]);
                 r[q] = rfma(-omega, y[q], w[q]);
             }
             if (small || rfma(-omega, rfma(-omega, a[2], rmul(T(2), a[3])), a[1]) <= tol2) break;
@@ -493,7 +498,7 @@ __device__ void bottom_solve(const Level<T> &L, T ih2, T *x, const T *f, T *scr,
         return;
     }
     // the fewest warps that hold the cells: their barriers cost less
-    const int per = (n + CT - 1) / CT, nthr = ((n + per - 1) / per + 31) & ~31;
+    const int per = n <= BOT_ONE ? 1 : 2, nthr = ((n + per - 1) / per + 31) & ~31;
     if (int(threadIdx.x) < nthr) {
         if (per == 1) team_bicgstab<T, 1>(L, x, f, scr, iters, singular, ih2, nthr);
         else team_bicgstab<T, BOT_REGS>(L, x, f, scr, iters, singular, ih2, nthr);
