@@ -44,6 +44,14 @@ constexpr int dist_min() {
     return sizeof(T) == sizeof(float) ? 1024 : 512;
 }
 
+// Largest level taken.  An FP64 warp instruction takes 64 clocks of its quarter of
+// the SM, so the 16 SMs of a cluster need 2.9 us for a colour pass of 32^3, more
+// than its launch over the whole GPU; FP32 is limited by the cells a CTA may own.
+template <typename T>
+constexpr int level_max() {
+    return sizeof(T) == sizeof(float) ? 65535 : 8192;
+}
+
 // Exact division of x < 2^16 by d < 2^16 as a multiply-high with the
 // precomputed m = ceil(2^32 / d) (the error x (m - 2^32/d) / 2^32 stays below
 // 1/d, so the floor is exact).
@@ -599,7 +607,7 @@ static bool plan_coarse(CoarseArgs<T> &A, const Level<T> *levs, int nl, int nc) 
     for (int l = 0; l < nl; l++) {
         const DGeom &g = levs[l].g;
         CoarseLevel<T> &C = A.lev[l];
-        if (g.N > 65535) return false;
+        if (g.N > level_max<T>()) return false;
         C.L = levs[l];
         C.dist = nc > 1 && l + 1 < nl && above_dist && g.N > dist_min<T>();
         above_dist = C.dist;
