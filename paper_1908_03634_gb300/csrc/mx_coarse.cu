@@ -250,10 +250,15 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
 #pragma unroll
         for (int q = 0; q < SL; q++)
             if (R.at[q]) {
-                T v[6];
-                neighbours(R, q, plane, v);
-                sm_at<T>(A.roff + R.at[q] - e0) =
-                    sm_at<T>(R.at[q] + df) - flux_sum(R.b[q], v, sm_at<T>(R.at[q])) * ih2;
+                T r = T(0);
+                // FP64, after a black pass: the black residuals are rounding (as in
+                // resid_restrict_red_kernel)
+                if (B == sizeof(float) || colour == 0 || passes == 0) {
+                    T v[6];
+                    neighbours(R, q, plane, v);
+                    r = sm_at<T>(R.at[q] + df) - flux_sum(R.b[q], v, sm_at<T>(R.at[q])) * ih2;
+                }
+                sm_at<T>(A.roff + R.at[q] - e0) = r;
             }
         team_sync(0, 2 * team);
         const int mx = nx >> 1, mxy = nxy >> 2, nown = (nxy * np) >> 3;

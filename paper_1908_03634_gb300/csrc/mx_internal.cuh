@@ -262,7 +262,8 @@ void k_prolong_batch(cudaStream_t s, const Level<float> *levs, const int4 *work,
 void k_finalize_residual_batch(cudaStream_t s, const double *partials, const int *off, const int *cnt, SolveState *st,
                                int nbox);
 template <typename T>
-void k_resid_restrict(cudaStream_t s, const Level<T> &fine, const Level<T> &coarse, int zcap = 8);
+void k_resid_restrict(cudaStream_t s, const Level<T> &fine, const Level<T> &coarse, int zcap = 8,
+                      int black_solved = 0);  // black_solved: e is fresh from a black pass
 template <typename T>
 void k_prolong(cudaStream_t s, const Level<T> &coarse, const Level<T> &fine, int zcap = 8);
 template <typename T>

@@ -343,6 +343,43 @@ __global__ void __launch_bounds__(SX *SY) resid_restrict_fine_kernel(Level<T> F,
     resid_restrict_fine_body(F, Cl, ih2, blockIdx.x, blockIdx.y, blockIdx.z, zcf);
 }
 
+// FP64, after a black pass: the black cells' residuals are rounding (their rows
+// were just solved), so only the red ones enter the means, in the same order.  A
+// thread takes the red cell of a pair (2I, 2I + 1) of one fine row and plane, so no
+// lane of an FP64 instruction is spent on black cells: half the FP64 work, which
+// bounds this kernel (128^3: 64 us with all cells).
+__global__ void __launch_bounds__(SX *SY) resid_restrict_red_kernel(Level<double> F, Level<double> Cl, double ih2,
+                                                                    int zcf) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ double sr[2][SY][SX];
+    const DGeom &g = F.g, &gc = Cl.g;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int I = blockIdx.x * SX + tx, j = blockIdx.y * SY + ty;
+    const bool act = I < gc.n[0] && j < g.n[1];
+    const int k0 = blockIdx.z * zcf, k1 = min(k0 + zcf, g.n[2]);  // k0 and zcf even
+    for (int k = k0; k < k1; k++) {
+        double r = 0.0;
+        if (act) {
+            const int i = 2 * I + ((j + k) & 1);
+            const long long c = i + (long long)g.n[0] * (j + (long long)g.n[1] * k);
+            double b[6], v[6];
+            face_coefs(F, i, j, k, c, b);
+            nb_vals(g, F.e, i, j, k, c, v);
+            r = F.f[c] - flux_sum(b, v, F.e[c]) * ih2;
+        }
+        sr[k & 1][ty][tx] = r;
+        if (k & 1) {
+            __syncthreads();
+            if (act && !(ty & 1)) {
+                const double sum = ((sr[0][ty][tx] + sr[0][ty + 1][tx]) + sr[1][ty][tx]) + sr[1][ty + 1][tx];
+                Cl.f[I + (long long)gc.n[0] * ((j >> 1) + (long long)gc.n[1] * (k >> 1))] = sum * 0.125;
+            }
+            __syncthreads();
+        }
+    }
+}
+
 template <typename T>
 __global__ void resid_restrict_kernel(Level<T> F, Level<T> Cl, T ih2, int zc) {
     pdl_trigger();
@@ -383,10 +420,20 @@ void k_resid_restrict_batch(cudaStream_t s, const Level<float> *levs, const int4
 }
 
 template <typename T>
-void k_resid_restrict(cudaStream_t s, const Level<T> &fine, const Level<T> &coarse, int zcap) {
+void k_resid_restrict(cudaStream_t s, const Level<T> &fine, const Level<T> &coarse, int zcap, int black_solved) {
     const double h = fine.g.h;
     const DGeom &g = fine.g;
     if (g.n[0] % 2 == 0 && g.n[1] % 2 == 0 && g.n[2] % 2 == 0) {
+        if constexpr (sizeof(T) == sizeof(double)) {
+            if (black_solved) {
+                const int bx = (coarse.g.n[0] + SX - 1) / SX, by = (g.n[1] + SY - 1) / SY;
+                int zcf = 16;
+                while (zcf > 2 && (long long)bx * by * ((g.n[2] + zcf - 1) / zcf) < 4 * 4 * 152) zcf >>= 1;
+                launch_pdl(resid_restrict_red_kernel, dim3(bx, by, (g.n[2] + zcf - 1) / zcf), dim3(SX, SY), 0, s, fine,
+                           coarse, 1.0 / (h * h), zcf);
+                return;
+            }
+        }
         // fine planes per block: even, halved until the grid fills the GPU a few times
         const long long bxy = (long long)((g.n[0] + SX - 1) / SX) * ((g.n[1] + SY - 1) / SY);
         int zcf = 16;
@@ -698,7 +745,7 @@ void k_residual_plain(cudaStream_t s, const Level<double> &L, const double *phi,
                                   const SolveState *, double *, int);                                            \
     template void k_update<T>(cudaStream_t, const DGeom &, double *, const T *, const SolveState *);            \
     template void k_rbgs<T>(cudaStream_t, const Level<T> &, int, int, int);                                      \
-    template void k_resid_restrict<T>(cudaStream_t, const Level<T> &, const Level<T> &, int);                  \
+    template void k_resid_restrict<T>(cudaStream_t, const Level<T> &, const Level<T> &, int, int);                \
     template void k_prolong<T>(cudaStream_t, const Level<T> &, const Level<T> &, int);                         \
     template void k_bottom<T>(cudaStream_t, const Level<T> &, T *, int, int);                                   \
     template void k_apply<T>(cudaStream_t, const Level<T> &, const T *, T *);                                   \

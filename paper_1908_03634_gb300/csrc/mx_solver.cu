@@ -248,7 +248,7 @@ void vcycle(cudaStream_t s, Hier<T> &H, int nu1, int nu2, int bot_iters, int sin
         }
         Level<T> Lc = L;
         Lc.e = cur[l];
-        k_resid_restrict(s, Lc, H.lev[l + 1], zcap);
+        k_resid_restrict(s, Lc, H.lev[l + 1], zcap, nu1 > 0);
         if (l == 0) {
             prof_end(pc, s, MX_PH_RESTRICT_FINE, 1);
             prof_begin(pc, s, MX_PH_COARSE);  // everything below the finest level
