@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "mx_coarse.cuh"
+#include "mx_rbgs.cuh"
 #include "mx_solver.cuh"
 #include "mx_stencil.cuh"
 
@@ -31,6 +32,7 @@ struct BatchPlan {
     // device-side descriptors
     void *mem = nullptr;
     Level<float> *d_levs = nullptr;  // [nbox * MX_MAXLEV]
+    Level<float> *d_swap = nullptr;  // the same with e and e2 exchanged
     DFBox *d_df = nullptr;           // [nbox]
     void *d_cargs = nullptr;         // coarse argument blocks
     SolveState *d_st = nullptr;      // [nbox]
@@ -38,6 +40,7 @@ struct BatchPlan {
     int *d_off = nullptr, *d_cnt = nullptr;
     int4 *d_work = nullptr;
     std::vector<WorkRange> rb, rr, pr;  // per level index
+    std::vector<int> sweep_zk;          // per level index: planes per chunk of single-pass sweeps (0: colour passes)
     std::vector<int> rr_zcf;            // per level index: fine planes per restriction tile (0: coarse tiles)
     WorkRange df;
     int nparts = 0;
@@ -113,10 +116,25 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
     B->rr.resize(B->maxdown);
     B->pr.resize(B->maxdown);
     B->rr_zcf.assign(B->maxdown, 0);
+    B->sweep_zk.assign(B->maxdown, 0);
     for (int l = 0; l < B->maxdown; l++) {
+        std::vector<DGeom> gl;
+        long long cells = 0;
+        bool sweeps = true;
+        for (int b = 0; b < nbox; b++)
+            if (l < B->lc[b]) {
+                gl.push_back(B->box[b]->H32.lev[l].g);
+                cells += gl.back().N;
+                sweeps = sweeps && rbgs_fused_ok(gl.back());
+            }
+        if (sweeps && cells >= SWEEP_MIN_CELLS) B->sweep_zk[l] = rbgs_sweep_zk(int(gl.size()), gl.data());
+        const int szk = B->sweep_zk[l];
         B->rb[l].off = int(work.size());
         for (int b = 0; b < nbox; b++)
-            if (l < B->lc[b]) add_grid(work, b, rbgs_grid(B->box[b]->H32.lev[l].g, ZC));
+            if (l < B->lc[b]) {
+                const DGeom &gb = B->box[b]->H32.lev[l].g;
+                add_grid(work, b, szk ? rbgs_sweep_grid(gb, szk) : rbgs_grid(gb, ZC));
+            }
         B->rb[l].n = int(work.size()) - B->rb[l].off;
         // residual + restriction: the fine-cell form when every box's level has even
         // extents, its fine planes per tile halved while the tiles fill the GPU less than
@@ -207,6 +225,7 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
     Bump dry{nullptr, 0};
     auto carve = [&](Bump &bm) {
         B->d_levs = bm.take<Level<float>>(levs.size());
+        B->d_swap = bm.take<Level<float>>(levs.size());
         B->d_df = bm.take<DFBox>(nbox);
         B->d_cargs = bm.take<char>(cargs.size());
         B->d_st = bm.take<SolveState>(nbox);
@@ -224,7 +243,10 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
     Bump real{(char *)B->mem, 0};
     carve(real);
     cudaStream_t s = c->stream;
+    std::vector<Level<float>> swapped = levs;
+    for (Level<float> &L : swapped) std::swap(L.e, L.e2);
     cudaMemcpyAsync(B->d_levs, levs.data(), sizeof(Level<float>) * levs.size(), cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(B->d_swap, swapped.data(), sizeof(Level<float>) * levs.size(), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(B->d_df, dfb.data(), sizeof(DFBox) * nbox, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(B->d_cargs, cargs.data(), cargs.size(), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(B->d_off, off.data(), sizeof(int) * nbox, cudaMemcpyHostToDevice, s);
@@ -245,7 +267,18 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
 // one V-cycle of every active box, then the fused update + residual and the
 // per-box convergence decision
 static void batch_body(cudaStream_t s, mx_ctx *c, BatchPlan &B, const mx_opts &o) {
+    // single-pass sweeps alternate between e and e2, starting so that the last one ends in e
+    auto sweep = [&](int l, int n) {  // the n-th of the level's nu1 + nu2 sweeps
+        k_rbgs_sweep_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, n == 0, (o.nu1 + o.nu2 - n) % 2 == 0,
+                           B.sweep_zk[l]);
+    };
     for (int l = 0; l < B.maxdown; l++) {
+        if (B.sweep_zk[l]) {
+            for (int q = 0; q < o.nu1; q++) sweep(l, q);
+            k_resid_restrict_batch(s, o.nu2 % 2 ? B.d_swap : B.d_levs, B.d_work + B.rr[l].off, B.rr[l].n, B.d_st, l,
+                                   B.rr_zcf[l]);
+            continue;
+        }
         for (int q = 0; q < o.nu1; q++) {
             k_rbgs_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, 0, q == 0);
             k_rbgs_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, 1, 0);
@@ -254,7 +287,14 @@ static void batch_body(cudaStream_t s, mx_ctx *c, BatchPlan &B, const mx_opts &o
     }
     k_coarse_vcycle_batch(s, B.d_cargs, B.d_st, B.nbox, B.coarse_smem);
     for (int l = B.maxdown - 1; l >= 0; l--) {
-        k_prolong_batch(s, B.d_levs, B.d_work + B.pr[l].off, B.pr[l].n, B.d_st, l);
+        if (B.sweep_zk[l]) {
+            // the prolongation on its own: applied on load it cost the batched sweep 300 us
+            // of 720 on 63 M cells, and the pass costs 110
+            k_prolong_batch(s, B.d_levs, o.nu2 % 2 ? B.d_swap : B.d_levs, B.d_work + B.pr[l].off, B.pr[l].n, B.d_st, l);
+            for (int q = 0; q < o.nu2; q++) sweep(l, o.nu1 + q);
+            continue;
+        }
+        k_prolong_batch(s, B.d_levs, B.d_levs, B.d_work + B.pr[l].off, B.pr[l].n, B.d_st, l);
         for (int q = 0; q < o.nu2; q++) {
             k_rbgs_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, 0, 0);
             k_rbgs_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, 1, 0);

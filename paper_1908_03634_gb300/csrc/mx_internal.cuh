@@ -257,8 +257,9 @@ void k_rbgs_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, in
 void k_resid_restrict_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, int nwork,
                             const SolveState *st, int level, int zcf);
 dim3 resid_restrict_fine_grid(const DGeom &fine, int zcf);
-void k_prolong_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, int nwork, const SolveState *st,
-                     int level);
+// fine: the descriptors whose e is corrected (levs, or those with e and e2 exchanged)
+void k_prolong_batch(cudaStream_t s, const Level<float> *levs, const Level<float> *fine, const int4 *work, int nwork,
+                     const SolveState *st, int level);
 void k_finalize_residual_batch(cudaStream_t s, const double *partials, const int *off, const int *cnt, SolveState *st,
                                int nbox);
 template <typename T>

@@ -485,17 +485,18 @@ __global__ void prolong_kernel(Level<T> Cl, Level<T> F, int zc) {
     prolong_body(Cl, F, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, threadIdx.y, zc);
 }
 
-__global__ void prolong_batch_kernel(const Level<float> *levs, const int4 *work, const SolveState *st, int level) {
+__global__ void prolong_batch_kernel(const Level<float> *levs, const Level<float> *fine, const int4 *work,
+                                     const SolveState *st, int level) {
     const int4 w = work[blockIdx.x];
     if (st[w.x].done) return;
     const Level<float> C = levs[w.x * MX_MAXLEV + level + 1];
-    const Level<float> F = levs[w.x * MX_MAXLEV + level];
+    const Level<float> F = fine[w.x * MX_MAXLEV + level];
     prolong_body(C, F, w.y, w.z, w.w, threadIdx.x, threadIdx.y, ZC);
 }
 
-void k_prolong_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, int nwork, const SolveState *st,
-                     int level) {
-    if (nwork > 0) prolong_batch_kernel<<<nwork, dim3(SX, SY), 0, s>>>(levs, work, st, level);
+void k_prolong_batch(cudaStream_t s, const Level<float> *levs, const Level<float> *fine, const int4 *work, int nwork,
+                     const SolveState *st, int level) {
+    if (nwork > 0) prolong_batch_kernel<<<nwork, dim3(SX, SY), 0, s>>>(levs, fine, work, st, level);
 }
 
 template <typename T>

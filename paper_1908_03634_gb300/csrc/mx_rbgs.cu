@@ -23,6 +23,8 @@
 // V-cycle level: no read of e); PROLONG = the input is e + P e_coarse
 // (piecewise-constant prolongation applied on load, the first sweep after the
 // coarse-grid correction).
+#include <algorithm>
+
 #include "mx_async.cuh"
 #include "mx_rbgs.cuh"
 #include "mx_stencil.cuh"
@@ -106,6 +108,8 @@ __device__ __forceinline__ void copy16(unsigned a, const void *src) {
 template <int MODE>
 struct March {
     const SweepArgs &A;
+    int bx, by;                   // tile
+    float h2;
     int nz, k0, k1;
     bool pz, in, out, xedge;
     unsigned mine;                // shared address of this lane's pair in the first stage's row wy
@@ -153,13 +157,13 @@ struct March {
     }
     // row of this warp and the staged place of bx at column nx
     __device__ __forceinline__ int hx_row() const {
-        return pos_of(int(blockIdx.y) * SW_TY - 1 + int(threadIdx.y), A.L.g.n[1], gper(A.L.g, 1)).at;
+        return pos_of(by * SW_TY - 1 + int(threadIdx.y), A.L.g.n[1], gper(A.L.g, 1)).at;
     }
     __device__ __forceinline__ bool row_in() const {
-        return pos_of(int(blockIdx.y) * SW_TY - 1 + int(threadIdx.y), A.L.g.n[1], gper(A.L.g, 1)).ok;
+        return pos_of(by * SW_TY - 1 + int(threadIdx.y), A.L.g.n[1], gper(A.L.g, 1)).ok;
     }
     __device__ __forceinline__ unsigned hx_dst() const {
-        return stage0() + ((SW_BX + threadIdx.y) * SW_RS + A.L.g.n[0] - int(blockIdx.x) * A.w + 4) * 4;
+        return stage0() + ((SW_BX + threadIdx.y) * SW_RS + A.L.g.n[0] - bx * A.w + 4) * 4;
     }
 
     __device__ __forceinline__ float parent(int o, int p) const {
@@ -218,7 +222,7 @@ struct March {
         }
         v[4] = em;
         v[5] = comp<C>(eu);
-        const float upd = gs_update(b, v, comp<C>(f), A.h2);
+        const float upd = gs_update(b, v, comp<C>(f), h2);
         const float red = in && (pz || (k >= 0 && k < nz)) ? upd : 0.f;
         // black cell of plane k-1, same column
         const float xl = left_of<C>(r1, r1), xr = right_of<C>(r1, r1);
@@ -237,7 +241,7 @@ struct March {
             v[3] = lds<P + 32>(ring);
             v[4] = r2;
             v[5] = red;
-            const float blk = gs_update(b, v, pf, A.h2);
+            const float blk = gs_update(b, v, pf, h2);
             *reinterpret_cast<float2 *>(to) = C ? make_float2(r1, blk) : make_float2(blk, r1);
             to = reinterpret_cast<float *>(reinterpret_cast<char *>(to) + plane);
         }
@@ -295,20 +299,18 @@ struct March {
 };
 
 template <int MODE>
-__global__ void __launch_bounds__(SW_THREADS, 2) rbgs_sweep_kernel(const __grid_constant__ SweepArgs A) {
-    pdl_trigger();
-    pdl_wait();
+__device__ __forceinline__ void sweep_body(const SweepArgs &A, int bx, int by, int bz) {
     const Level<float> &L = A.L;
     const DGeom &g = L.g;
     const int nx = g.n[0], ny = g.n[1], nxy = nx * ny;
     const bool px = gper(g, 0), py = gper(g, 1);
     const int lane = threadIdx.x, wy = threadIdx.y, tid = lane + 32 * wy;
-    const int x0 = blockIdx.x * A.w, j0 = blockIdx.y * SW_TY;
-    March<MODE> m{A};
+    const int x0 = bx * A.w, j0 = by * SW_TY;
+    March<MODE> m{A, bx, by, A.h2};
     m.plane = unsigned(nxy) * 4u;
     m.nz = g.n[2];
     m.pz = gper(g, 2);
-    m.k0 = blockIdx.z * A.zk;
+    m.k0 = bz * A.zk;
     m.k1 = min(m.k0 + A.zk, m.nz);
     const int i = x0 - 2 + 2 * lane, j = j0 - 1 + wy;
     const Pos x = pos_of(i, nx, px), y = pos_of(j, ny, py);
@@ -369,6 +371,52 @@ __global__ void __launch_bounds__(SW_THREADS, 2) rbgs_sweep_kernel(const __grid_
     else m.template run<0>();
 }
 
+template <int MODE>
+__global__ void __launch_bounds__(SW_THREADS, 2) rbgs_sweep_kernel(const __grid_constant__ SweepArgs A) {
+    pdl_trigger();
+    pdl_wait();
+    sweep_body<MODE>(A, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// tiles of equal width, a multiple of 4
+__host__ __device__ inline int sweep_width(const DGeom &g) {
+    const int tx = (g.n[0] + SW_WMAX - 1) / SW_WMAX;
+    return ((g.n[0] + tx - 1) / tx + 3) / 4 * 4;
+}
+
+// batched: work[blockIdx.x] = (box, tile x, tile y, chunk of zk planes); to_e2: from
+// e into e2, else from e2 into e
+template <int MODE>
+__global__ void __launch_bounds__(SW_THREADS, 2)
+    rbgs_sweep_batch_kernel(const Level<float> *levs, const int4 *work, const SolveState *st, int level, int to_e2,
+                            int zk) {
+    const int4 q = work[blockIdx.x];
+    if (st[q.x].done) return;
+    __shared__ SweepArgs A;
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        A.L = levs[q.x * MX_MAXLEV + level];
+        A.ein = to_e2 ? A.L.e : A.L.e2;
+        A.eout = to_e2 ? A.L.e2 : A.L.e;
+        A.h2 = float(A.L.g.h * A.L.g.h);
+        A.w = sweep_width(A.L.g);
+        A.zk = zk;
+    }
+    __syncthreads();
+    sweep_body<MODE>(A, q.y, q.z, q.w);
+}
+
+dim3 rbgs_sweep_grid(const DGeom &g, int zk) {
+    const int w = sweep_width(g);
+    return dim3((g.n[0] + w - 1) / w, (g.n[1] + SW_TY - 1) / SW_TY, (g.n[2] + zk - 1) / zk);
+}
+
+void k_rbgs_sweep_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, int nwork, const SolveState *st,
+                        int level, int zero, int to_e2, int zk) {
+    if (nwork <= 0) return;
+    auto k = zero ? rbgs_sweep_batch_kernel<RB_ZERO> : rbgs_sweep_batch_kernel<RB_PLAIN>;
+    k<<<nwork, dim3(32, SW_ROWS), SW_SMEM, s>>>(levs, work, st, level, to_e2, zk);
+}
+
 bool rbgs_fused_ok(const DGeom &g) {
     // rows in 16-byte chunks; a periodic axis wraps at most once and keeps the colour
     if (g.n[0] % 4 || g.n[0] < 32 || g.n[1] < 4 || g.n[2] < 4) return false;
@@ -378,12 +426,37 @@ bool rbgs_fused_ok(const DGeom &g) {
 }
 
 cudaError_t rbgs_init() {
-    cudaError_t e = cudaFuncSetAttribute(rbgs_sweep_kernel<RB_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SW_SMEM));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(rbgs_sweep_kernel<RB_ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SW_SMEM));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(rbgs_sweep_kernel<RB_PROLONG>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SW_SMEM));
-    return e;
+    const void *kernels[] = {(const void *)rbgs_sweep_kernel<RB_PLAIN>, (const void *)rbgs_sweep_kernel<RB_ZERO>,
+                             (const void *)rbgs_sweep_kernel<RB_PROLONG>, (const void *)rbgs_sweep_batch_kernel<RB_PLAIN>,
+                             (const void *)rbgs_sweep_batch_kernel<RB_ZERO>};
+    for (const void *k : kernels) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SW_SMEM));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// The planes per chunk that make the fewest steps in a row: whole waves of two
+// blocks per SM times the planes a block walks (its chunk, one on either side, and
+// the time to the first plane).
+int rbgs_sweep_zk(int nbox, const DGeom *g) {
+    int nz = 0, zk = 1;
+    for (int b = 0; b < nbox; b++) nz = std::max(nz, g[b].n[2]);
+    long long best = -1;
+    for (int c = 1; c <= nz && c <= 64; c++) {
+        const int z = (nz + c - 1) / c;
+        long long blocks = 0;
+        for (int b = 0; b < nbox; b++) {
+            const dim3 gr = rbgs_sweep_grid(g[b], z);
+            blocks += (long long)gr.x * gr.y * gr.z;
+        }
+        const long long cost = (blocks + 2 * 152 - 1) / (2 * 152) * (z + 3);
+        if (best < 0 || cost < best) {
+            best = cost;
+            zk = z;
+        }
+    }
+    return zk;
 }
 
 void k_rbgs_fused(cudaStream_t s, const Level<float> &L, const float *ein, float *eout, int mode,
@@ -397,21 +470,9 @@ void k_rbgs_fused(cudaStream_t s, const Level<float> &L, const float *ein, float
     A.ncx = coarse ? coarse->g.n[0] : 0;
     A.ncy = coarse ? coarse->g.n[1] : 0;
     A.h2 = float(g.h * g.h);
-    // tiles of equal width; the z chunks that make the fewest steps in a row: whole
-    // waves of two blocks per SM times the planes a block walks (its chunk, one on
-    // either side, and the time to the first plane)
-    const int tx = (g.n[0] + SW_WMAX - 1) / SW_WMAX, ty = (g.n[1] + SW_TY - 1) / SW_TY;
-    A.w = ((g.n[0] + tx - 1) / tx + 3) / 4 * 4;
-    long long best = -1;
-    for (int c = 1; c <= g.n[2] && c <= 64; c++) {
-        const int zk = (g.n[2] + c - 1) / c, used = (g.n[2] + zk - 1) / zk;
-        const long long cost = ((long long)tx * ty * used + 2 * 152 - 1) / (2 * 152) * (zk + 3);
-        if (best < 0 || cost < best) {
-            best = cost;
-            A.zk = zk;
-        }
-    }
-    const dim3 grid((g.n[0] + A.w - 1) / A.w, ty, (g.n[2] + A.zk - 1) / A.zk);
+    A.w = sweep_width(g);
+    A.zk = rbgs_sweep_zk(1, &g);
+    const dim3 grid = rbgs_sweep_grid(g, A.zk);
     auto k = mode == RB_ZERO ? rbgs_sweep_kernel<RB_ZERO>
              : mode == RB_PROLONG ? rbgs_sweep_kernel<RB_PROLONG> : rbgs_sweep_kernel<RB_PLAIN>;
     launch_pdl(k, grid, dim3(32, SW_ROWS), SW_SMEM, s, A);

@@ -53,7 +53,14 @@ __device__ __forceinline__ float gs_update(const float b[6], const float v[6], f
     return gs_update(b, v, f, h2, gs_inverse(b));
 }
 
-// Whether the single-pass sweep supports this level (n_x even, periodic extents >= 2).
+// FP32 levels of at least so many cells smooth by single-pass sweeps.  A sweep moves
+// half the bytes of two colour passes but takes more of the SMs' shared-memory
+// pipe, so the line lies where e, f and the coefficients (20 B per cell) outgrow the
+// 126 MB L2: measured, 256^3 96 us a sweep against 112 us, 160x192x224 42 against
+// 46, and 128^3, out of L2, 21 against 18.
+constexpr long long SWEEP_MIN_CELLS = 6LL << 20;
+
+// Whether the single-pass sweep supports this level (n_x a multiple of 4, at least 32).
 bool rbgs_fused_ok(const DGeom &g);
 
 // Allow the sweep kernels their shared memory (once per device, outside any capture).
@@ -63,3 +70,11 @@ cudaError_t rbgs_init();
 // RB_PROLONG: e_in + piecewise-constant prolongation of coarse->e).
 void k_rbgs_fused(cudaStream_t s, const Level<float> &L, const float *ein, float *eout, int mode,
                   const Level<float> *coarse);
+
+// The same over a batch: work entries (box, tile x, tile y, chunk) of
+// rbgs_sweep_grid(level geometry, zk), zk from rbgs_sweep_zk over the boxes; e -> e2
+// (to_e2) or e2 -> e
+dim3 rbgs_sweep_grid(const DGeom &g, int zk);
+int rbgs_sweep_zk(int nbox, const DGeom *g);
+void k_rbgs_sweep_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, int nwork, const SolveState *st,
+                        int level, int zero, int to_e2, int zk);

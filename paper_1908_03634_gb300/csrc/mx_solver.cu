@@ -196,13 +196,7 @@ void destroy_plans(mx_ctx *c) {
 //  * other levels above the coarse end: two-pass colour kernels in place;
 //  * the coarse end (the levels that fit one cluster's shared memory, down to the
 //    bottom): one launch; without such a level, a BiCGStab bottom kernel.
-//
-// A sweep moves half the bytes of two colour passes but takes more of the SMs'
-// shared-memory pipe, so the line lies where e, f and the coefficients (20 B per
-// cell) outgrow the 126 MB L2: measured, 256^3 96 us a sweep against 112 us,
-// 160x192x224 42 against 46, and 128^3, out of L2, 21 against 18.
 constexpr long long FUSED_MIN_CELLS = 1LL << 18;
-constexpr long long SWEEP_MIN_CELLS = 6LL << 20;
 
 template <typename T>
 int coarse_start(const Hier<T> &H, int clustered) {

@@ -51,3 +51,32 @@ def test_sweep_bits(mx, ctx, n, bc, nu):
         assert info["vcycles"] == 2 and np.isfinite(info["rel_resid"])
         out.append(phi.cpu().numpy())
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nu", [(1, 3), (2, 2)])
+def test_batched_sweeps_equal_single_colour_passes(mx, ctx, nu):
+    """A batch large enough for single-pass sweeps on its finest level (6 M cells)
+    against single solves of its boxes, which run colour passes: the same bits."""
+    boxes = [((128, 128, 128), (P, P, N)), ((160, 128, 144), (P, D, N)), ((64, 64, 64), (D, D, D)),
+             ((128, 112, 136), (N, P, P))]
+    rng = np.random.default_rng(4)
+    cuda = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    gs, rho, beta0, sbar, us = [], [], [], [], []
+    for n, bc in boxes:
+        g = W.Geom(n, 1.0 / n[0], bc, bc)
+        cs = mx.cell_shape(g)
+        gs.append(g)
+        rho.append(cuda(np.exp(0.5 * rng.standard_normal(cs))))
+        beta0.append(cuda(np.exp(0.5 * rng.standard_normal(cs))))
+        sbar.append(cuda(rng.standard_normal(cs)))
+        us.append(W._periodic_faces(g, [torch.from_numpy(rng.standard_normal(g.face_shape(d))) for d in range(3)]))
+    assert sum(n[0] * n[1] * n[2] for n, _ in boxes) >= 6 << 20
+    opts = mx.default_opts(nu1=nu[0], nu2=nu[1], max_outer=2)
+    allow = (mx.MX_OK, mx.MX_ERR_NOCONV)
+    phi = [torch.zeros_like(r) for r in rho]
+    mx.mx_mac_project_batched(ctx, gs, *[[cuda(u[d].numpy()) for u in us] for d in range(3)], rho, beta0, sbar, phi,
+                              opts, allow=allow)
+    for b, g in enumerate(gs):
+        one = torch.zeros_like(rho[b])
+        mx.mx_mac_project(ctx, g, *[cuda(t.numpy()) for t in us[b]], rho[b], beta0[b], sbar[b], one, opts, allow=allow)
+        assert torch.equal(one, phi[b])
