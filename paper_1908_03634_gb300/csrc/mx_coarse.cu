@@ -117,7 +117,7 @@ __device__ __forceinline__ void remote_load(unsigned a, double &v) {
 // threads (whole warps; a small level's barriers then cost less).
 __device__ __forceinline__ void team_sync(int dist, int nthr) {
     if (dist) cluster_sync();
-    else asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+    else asm volatile("barrier.sync 1, %0;" ::"r"(nthr) : "memory");
 }
 
 // the 6 face coefficients of in-box cell (i,j,k) = c with 32-bit indexing (the

@@ -194,7 +194,7 @@ struct March {
     __device__ __forceinline__ void step(int k) {
         cp_async_wait<1>();  // plane k+1 has arrived (this thread's part)
         // warps of odd and even rows run different copies of this
-        asm volatile("bar.sync 0;" ::: "memory");
+        asm volatile("barrier.sync 0;" ::: "memory");
         fetch<(S + 3) % SW_STAGES>(k + 3);
         constexpr int G = S * SW_STAGE, U = (S + 1) % SW_STAGES * SW_STAGE;
         const float2 bx = lds2<G + SW_BX * SW_RS>(mine), f = lds2<G + SW_F * SW_RS>(mine);
@@ -279,7 +279,7 @@ struct March {
         fetch<0>(first);
         fetch<1>(first + 1);
         cp_async_wait<1>();
-        asm volatile("bar.sync 0;" ::: "memory");
+        asm volatile("barrier.sync 0;" ::: "memory");
         em = comp<C>(old_pair<3>(MODE == RB_PROLONG ? parent(cc, first - 1) : 0.f));
         e0 = old_pair<0>(MODE == RB_PROLONG ? parent(cc, first) : 0.f);
         bz0 = lds2<SW_BZ * SW_RS>(mine);

@@ -15,7 +15,8 @@ struct TeamSum {
     int nthr, turn = 0;
 
     __device__ __forceinline__ TeamSum(T (*r)[4][32], int n) : red(r), nthr(n) {}
-    __device__ __forceinline__ void barrier() const { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); }
+    // (the form without .aligned: warps may arrive in parts, after a divergent branch)
+    __device__ __forceinline__ void barrier() const { asm volatile("barrier.sync 1, %0;" ::"r"(nthr) : "memory"); }
     static __device__ __forceinline__ T group_sum(T k) {
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
