@@ -113,11 +113,10 @@ __device__ __forceinline__ void remote_load(unsigned a, double &v) {
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
 }
 
-// The threads that hold a level's cells: the cluster, or the block's first nthr
-// threads (whole warps; a small level's barriers then cost less).
-__device__ __forceinline__ void team_sync(int dist, int nthr) {
+// The threads that hold a level's cells: the cluster or the block.
+__device__ __forceinline__ void level_sync(int dist) {
     if (dist) cluster_sync();
-    else asm volatile("barrier.sync 1, %0;" ::"r"(nthr) : "memory");
+    else __syncthreads();
 }
 
 // the 6 face coefficients of in-box cell (i,j,k) = c with 32-bit indexing (the
@@ -170,7 +169,7 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
     const int nx = g.n[0], ny = g.n[1], nxy = nx * ny, dist = C.dist;
     const int k0 = rank * C.pp, np = max(0, min(C.pp, g.n[2] - k0)), half = (nxy * np) >> 1;
     const int team = dist ? CT / 2 : ((half + SL - 1) / SL + 31) & ~31;  // threads per colour
-    if (int(threadIdx.x) >= 2 * team) return;
+    const bool works = int(threadIdx.x) < 2 * team;
     const int colour = int(threadIdx.x) >= team;
     const int e0 = C.eoff + nxy * B, plane = nxy * B, df = C.foff - e0;
     Cells<T, SL> R;
@@ -185,7 +184,7 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
             const int m = int(threadIdx.x) - colour * team + team * q;
             R.at[q] = 0;
             R.push[q] = 0;
-            if (m < half) {
+            if (works && m < half) {
                 const int r = fdiv(m, C.dh);  // row j + n1 p
                 const int p = fdiv(r, C.d1);
                 const int j = r - p * ny, k = k0 + p;
@@ -226,7 +225,7 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
                 sm_at<T>(R.at[q]) = v;
                 if (R.push[q]) remote_store(R.push[q], v);
             }
-        team_sync(dist, 2 * team);
+        level_sync(dist);
     }
     const T h2 = C.h2;
     const int passes = 2 * (up ? A.nu2 : A.nu1);
@@ -243,7 +242,7 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
                     if (R.push[q]) remote_store(R.push[q], e);
                 }
         }
-        team_sync(dist, 2 * team);
+        level_sync(dist);
     }
     if (!up) {  // the level below: right-hand side = means of the 8 residuals
         const T ih2 = C.ih2;
@@ -260,9 +259,9 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
                 }
                 sm_at<T>(A.roff + R.at[q] - e0) = r;
             }
-        team_sync(0, 2 * team);
+        __syncthreads();
         const int mx = nx >> 1, mxy = nxy >> 2, nown = (nxy * np) >> 3;
-        for (int t = threadIdx.x; t < nown; t += 2 * team) {
+        for (int t = threadIdx.x; t < nown; t += CT) {
             const int r = fdiv(t, F.d0);
             const int P = fdiv(r, F.d1);
             const int I = t - r * mx, J = r - P * int(F.d1.d), K = (k0 >> 1) + P;
@@ -298,9 +297,8 @@ __device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b)
 // The operations are rounded explicitly, so the single and the batched kernel
 // agree bit for bit.
 template <typename T, int B>
-__device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular,
+__device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular,
                                               T ih2, int nthr) {
-    __shared__ T red[2][4][32];
     const int n = int(L.g.N), nx = L.g.n[0], ny = L.g.n[1], nz = L.g.n[2], nxy = nx * ny;
     T b[B][6], den[B], dinv[B], xv[B], r[B], r0[B], p[B], v[B];
     unsigned nb[B][3];
@@ -330,7 +328,7 @@ __device__ __forceinline__ void team_bicgstab(const Level<T> &L, T *x, const T *
         den[q] = radd(radd(radd(b[q][0], b[q][1]), radd(b[q][2], b[q][3])), radd(b[q][4], b[q][5]));
         dinv[q] = den[q] != T(0) ? rinv(den[q]) : T(0);
     }
-    TeamSum<T> team(red, nthr);
+    TeamSum<T> team(S, nthr);
     const T inv_n = T(1) / T(n);
     T mean = T(0), rho1 = T(0), rho = T(1), alpha = T(1), omega = T(1), tol2 = T(0);
     // step -1: the mean of f and ||f - mean||^2; then the iterations
@@ -503,18 +501,25 @@ __device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int it
     }
 }
 
+// cells per thread, and threads, of a bottom solve in registers: the fewest warps that
+// hold the cells (their barriers cost less); 0 threads: too large
+__device__ __forceinline__ int bottom_per(int n) { return n <= BOT_ONE ? 1 : BOT_REGS; }
+__device__ __forceinline__ int bottom_threads(int n) {
+    const int per = bottom_per(n);
+    return n > BOT_REGS * CT ? 0 : ((n + per - 1) / per + 31) & ~31;
+}
+
 template <typename T>
-__device__ void bottom_solve(const Level<T> &L, T ih2, T *x, const T *f, T *scr, int iters, int singular) {
+__device__ void bottom_solve(TeamShared<T> &S, const Level<T> &L, T ih2, T *x, const T *f, T *scr, int iters, int singular) {
     const int n = int(L.g.N);
-    if (n > BOT_REGS * CT) {
+    const int per = bottom_per(n), nthr = bottom_threads(n);
+    if (!nthr) {
         cta_bicgstab(L, x, f, scr, iters, singular, ih2);
         return;
     }
-    // the fewest warps that hold the cells: their barriers cost less
-    const int per = n <= BOT_ONE ? 1 : 2, nthr = ((n + per - 1) / per + 31) & ~31;
     if (int(threadIdx.x) < nthr) {
-        if (per == 1) team_bicgstab<T, 1>(L, x, f, scr, iters, singular, ih2, nthr);
-        else team_bicgstab<T, BOT_REGS>(L, x, f, scr, iters, singular, ih2, nthr);
+        if (per == 1) team_bicgstab<T, 1>(S, L, x, f, scr, iters, singular, ih2, nthr);
+        else team_bicgstab<T, BOT_REGS>(S, L, x, f, scr, iters, singular, ih2, nthr);
     }
     __syncthreads();
 }
@@ -522,6 +527,8 @@ __device__ void bottom_solve(const Level<T> &L, T ih2, T *x, const T *f, T *scr,
 template <typename T, int SLMAX>
 __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &A, int rank) {
     constexpr int B = sizeof(T);
+    __shared__ TeamShared<T> bottom;
+    if (threadIdx.x == 0 && rank == 0) team_init(bottom, max(32, bottom_threads(int(A.lev[A.nl - 1].L.g.N))));
     for (int q = threadIdx.x * B; q < A.roff; q += CT * B) sm_at<T>(q) = T(0);
     __syncthreads();
     const int first = rank * A.lev[0].pp, nxy0 = int(A.lev[0].L.g.nxy);  // this CTA's planes of the first level
@@ -535,7 +542,7 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &A, int rank) {
         if (step == nb) {
             const CoarseLevel<T> &C = A.lev[nb];
             if (rank == 0)
-                bottom_solve(C.L, C.ih2, &sm_at<T>(C.eoff + int(C.L.g.nxy) * B), &sm_at<T>(C.foff), &sm_at<T>(A.roff),
+                bottom_solve(bottom, C.L, C.ih2, &sm_at<T>(C.eoff + int(C.L.g.nxy) * B), &sm_at<T>(C.foff), &sm_at<T>(A.roff),
                              A.bot_iters, A.singular);
             continue;
         }

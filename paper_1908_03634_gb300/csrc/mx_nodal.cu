@@ -572,13 +572,17 @@ __device__ void nd_wmean0(const NGeom &g, T *x) {
 // per V-cycle when every product re-read the 8 cells and every sum was its own
 // block-wide reduction.
 template <typename T>
-__device__ __forceinline__ void nd_team_bicgstab(const NLevel<T> &L, int iters, int nthr) {
-    __shared__ T vec[2][NBT + 1];
-    __shared__ float red[2][4][32];
+struct NdTeam {
+    TeamShared<float> team;
+    T vec[2][NBT + 1];
+};
+template <typename T>
+__device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &L, int iters, int nthr) {
+    const unsigned vec[2] = {unsigned(__cvta_generic_to_shared(S.vec[0])), unsigned(__cvta_generic_to_shared(S.vec[1]))};
     const NGeom &g = L.g;
     const int n = int(g.M), q = threadIdx.x;
-    TeamSum<float> team(red, nthr);
-    if (q < 2) vec[q][n] = T(0);
+    TeamSum<float> team(S.team, nthr);
+    if (q < 2) team_put(vec[0] + (q * (NBT + 1) + n) * unsigned(sizeof(T)), T(0));
     T coef[20], den = T(0), inv = T(0), dinv = T(0);
     unsigned nb[10];
     float w = 0.f;
@@ -637,13 +641,14 @@ __device__ __forceinline__ void nd_team_bicgstab(const NLevel<T> &L, int iters, 
 #pragma unroll 1
             for (int h = 0; h < 2; h++) {  // y = L u: v = L p, then t = L s
                 const T uh = u * dinv;
-                if (q < n) vec[h][q] = uh;
+                const unsigned vh = h ? vec[1] : vec[0];
+                if (q < n) team_put(vh + q * unsigned(sizeof(T)), uh);
                 team.barrier();
                 T n0 = T(0), n1 = T(0);
 #pragma unroll
                 for (int m = 0; m < 10; m++) {
-                    n0 += coef[2 * m] * vec[h][nb[m] & 0xffffu];
-                    n1 += coef[2 * m + 1] * vec[h][nb[m] >> 16];
+                    n0 += coef[2 * m] * team_get(vh + (nb[m] & 0xffffu) * unsigned(sizeof(T)), T(0));
+                    n1 += coef[2 * m + 1] * team_get(vh + (nb[m] >> 16) * unsigned(sizeof(T)), T(0));
                 }
                 y = ((n0 + n1) - den * uh) * inv;
                 const float wy = w * float(y), fu = float(u), fy = float(y);
@@ -683,8 +688,11 @@ __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int
     const NGeom &g = L.g;
     const int n = int(g.M);
     if (n <= NBT) {
+        __shared__ NdTeam<T> S;
         const int nthr = (n + 31) & ~31;
-        if (int(threadIdx.x) < nthr) nd_team_bicgstab(L, iters, nthr);
+        if (threadIdx.x == 0) team_init(S.team, nthr);
+        __syncthreads();
+        if (int(threadIdx.x) < nthr) nd_team_bicgstab(S, L, iters, nthr);
         return;
     }
     T *x = L.e, *r = scr, *r0 = scr + n, *p = scr + 2 * n, *v = scr + 3 * n, *sv = scr + 4 * n, *tv = scr + 5 * n;
