@@ -178,3 +178,27 @@ def test_split_errors(mx, ctx):
     with pytest.raises(mx.MXError) as e:  # radius table beyond 2^26 entries
         mx.mx_add_w0_faces(ctx, g, 1, (1 << 20, 0, 0), torch.zeros(9, dtype=torch.float64, device=DEV), out, *u)
     assert e.value.status == mx.MX_ERR_ARG
+
+
+@pytest.mark.parametrize("n,c", [((700, 6, 5), (350, 3, 2)), ((517, 4, 3), (258, -2, 7)), ((2, 9, 1), (1, 4, 0))])
+def test_split_wide_and_narrow_rows(mx, ctx, n, c):
+    """rows of more column pairs than a block has threads, odd rows, and plane counts on
+    either side of a thread's four: the bounds of the tests above (2^-40 of the values
+    for the bracket, 1e-12 for the faces)"""
+    g = W.Geom(n, 1.0 / 64, (N, N, N), (N, N, N))
+    rng = np.random.default_rng(11)
+    S = rng.standard_normal(O.cell_shape(g)) + np.linspace(1, 3, n[0])
+    want = O.subtract_lateral_average(g, 1, c, S)
+    out = torch.empty(O.cell_shape(g), dtype=torch.float64, device=DEV)
+    mx.mx_subtract_lateral_average(ctx, g, 1, c, dev(S), out)
+    r = np.arange(61) * (g.dx / 2)
+    w0 = np.sin(9.0 * r) + 0.3 * r
+    u = [rng.standard_normal(O.face_shape(g, d)) for d in range(3)]
+    faces = O.add_w0_faces(g, True, c, r, w0, u)
+    ud = [dev(x) for x in u]
+    mx.mx_add_w0_faces(ctx, g, 1, c, dev(r), dev(w0), *ud)
+    torch.cuda.synchronize()
+    assert np.abs(out.cpu().numpy() - want).max() <= 2.0**-40 * np.abs(S).max()
+    scale = max(np.abs(x).max() for x in u) + np.abs(w0).max()
+    for d in range(3):
+        assert np.abs(ud[d].cpu().numpy() - faces[d]).max() <= 1e-12 * scale
