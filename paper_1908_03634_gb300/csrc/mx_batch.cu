@@ -41,6 +41,7 @@ struct BatchPlan {
     int4 *d_work = nullptr;
     std::vector<WorkRange> rb, rr, pr;  // per level index
     std::vector<int> sweep_zk;          // per level index: planes per chunk of single-pass sweeps (0: colour passes)
+    std::vector<char> rr_quad;          // per level index: restriction by 2 x 2 columns per thread
     std::vector<int> rr_zcf;            // per level index: fine planes per restriction tile (0: coarse tiles)
     WorkRange df;
     int nparts = 0;
@@ -116,6 +117,7 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
     B->rr.resize(B->maxdown);
     B->pr.resize(B->maxdown);
     B->rr_zcf.assign(B->maxdown, 0);
+    B->rr_quad.assign(B->maxdown, 0);
     B->sweep_zk.assign(B->maxdown, 0);
     for (int l = 0; l < B->maxdown; l++) {
         std::vector<DGeom> gl;
@@ -139,31 +141,36 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
         // residual + restriction: the fine-cell form when every box's level has even
         // extents, its fine planes per tile halved while the tiles fill the GPU less than
         // four times at four blocks per SM (as for a single box)
-        bool even = true;
+        bool even = true, quad = true;
+        cells = 0;
         for (int b = 0; b < nbox; b++)
             if (l < B->lc[b]) {
                 const DGeom &gf = B->box[b]->H32.lev[l].g;
                 even = even && gf.n[0] % 2 == 0 && gf.n[1] % 2 == 0 && gf.n[2] % 2 == 0;
+                quad = quad && resid_restrict_quad_ok(B->box[b]->H32.lev[l]);
+                cells += gf.N;
             }
+        quad = quad && cells >= RESTRICT_QUAD_MIN;
         int zcf = 0;
         if (even) {
             auto tiles = [&](int z) {
                 long long t = 0;
                 for (int b = 0; b < nbox; b++)
                     if (l < B->lc[b]) {
-                        const dim3 gr = resid_restrict_fine_grid(B->box[b]->H32.lev[l].g, z);
+                        const dim3 gr = resid_restrict_fine_grid(B->box[b]->H32.lev[l].g, z, quad);
                         t += (long long)gr.x * gr.y * gr.z;
                     }
                 return t;
             };
             zcf = 16;
-            while (zcf > 2 && tiles(zcf) < 4 * 4 * 152) zcf >>= 1;
+            while (zcf > 2 && tiles(zcf) < (quad ? 8 : 4) * 4 * 152) zcf >>= 1;
         }
         B->rr_zcf[l] = zcf;
+        B->rr_quad[l] = quad;
         B->rr[l].off = int(work.size());
         for (int b = 0; b < nbox; b++)
             if (l < B->lc[b])
-                add_grid(work, b, zcf ? resid_restrict_fine_grid(B->box[b]->H32.lev[l].g, zcf)
+                add_grid(work, b, zcf ? resid_restrict_fine_grid(B->box[b]->H32.lev[l].g, zcf, quad)
                                       : stencil_grid_zc(B->box[b]->H32.lev[l + 1].g, ZC));
         B->rr[l].n = int(work.size()) - B->rr[l].off;
         B->pr[l].off = int(work.size());
@@ -276,14 +283,15 @@ static void batch_body(cudaStream_t s, mx_ctx *c, BatchPlan &B, const mx_opts &o
         if (B.sweep_zk[l]) {
             for (int q = 0; q < o.nu1; q++) sweep(l, q);
             k_resid_restrict_batch(s, o.nu2 % 2 ? B.d_swap : B.d_levs, B.d_work + B.rr[l].off, B.rr[l].n, B.d_st, l,
-                                   B.rr_zcf[l]);
+                                   B.rr_zcf[l], B.rr_quad[l]);
             continue;
         }
         for (int q = 0; q < o.nu1; q++) {
             k_rbgs_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, 0, q == 0);
             k_rbgs_batch(s, B.d_levs, B.d_work + B.rb[l].off, B.rb[l].n, B.d_st, l, 1, 0);
         }
-        k_resid_restrict_batch(s, B.d_levs, B.d_work + B.rr[l].off, B.rr[l].n, B.d_st, l, B.rr_zcf[l]);
+        k_resid_restrict_batch(s, B.d_levs, B.d_work + B.rr[l].off, B.rr[l].n, B.d_st, l, B.rr_zcf[l],
+                                   B.rr_quad[l]);
     }
     k_coarse_vcycle_batch(s, B.d_cargs, B.d_st, B.nbox, B.coarse_smem);
     for (int l = B.maxdown - 1; l >= 0; l--) {

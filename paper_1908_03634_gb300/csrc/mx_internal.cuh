@@ -255,8 +255,13 @@ void k_rbgs_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, in
 // zcf > 0: the fine-cell form, work entries are tiles of resid_restrict_fine_grid(level's
 // geometry, zcf) (every box's level has even extents); 0: tiles of the coarse level
 void k_resid_restrict_batch(cudaStream_t s, const Level<float> *levs, const int4 *work, int nwork,
-                            const SolveState *st, int level, int zcf);
-dim3 resid_restrict_fine_grid(const DGeom &fine, int zcf);
+                            const SolveState *st, int level, int zcf, bool quad);
+dim3 resid_restrict_fine_grid(const DGeom &fine, int zcf, bool quad);
+// FP32 levels (batches: the boxes' levels together) of at least so many cells restrict
+// by 2 x 2 columns per thread where the level allows it; smaller ones need the four
+// times as many threads of one cell each
+constexpr long long RESTRICT_QUAD_MIN = 1LL << 20;
+bool resid_restrict_quad_ok(const Level<float> &fine);
 // fine: the descriptors whose e is corrected (levs, or those with e and e2 exchanged)
 void k_prolong_batch(cudaStream_t s, const Level<float> *levs, const Level<float> *fine, const int4 *work, int nwork,
                      const SolveState *st, int level);

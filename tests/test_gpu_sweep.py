@@ -80,3 +80,33 @@ def test_batched_sweeps_equal_single_colour_passes(mx, ctx, nu):
         one = torch.zeros_like(rho[b])
         mx.mx_mac_project(ctx, g, *[cuda(t.numpy()) for t in us[b]], rho[b], beta0[b], sbar[b], one, opts, allow=allow)
         assert torch.equal(one, phi[b])
+
+
+def test_restriction_by_columns_equals_one_cell_per_thread(mx, ctx):
+    """A batch of a million cells restricts by 2 x 2 columns per thread, single solves of
+    its boxes by one cell per thread: the same bits.  Rows of one and two tiles of 64
+    and a few pairs more, rows of blocks and chunks of planes that end early, every
+    kind of face on every axis."""
+    boxes = [((132, 24, 28), (D, P, N)), ((68, 36, 40), (P, N, D)), ((36, 132, 20), (N, D, P)),
+             ((128, 8, 72), (P, P, P)), ((96, 96, 96), (P, P, N))]
+    assert sum(n[0] * n[1] * n[2] for n, _ in boxes) >= 1 << 20 > max(n[0] * n[1] * n[2] for n, _ in boxes)
+    rng = np.random.default_rng(6)
+    cuda = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    gs, rho, beta0, sbar, us = [], [], [], [], []
+    for n, bc in boxes:
+        g = W.Geom(n, 1.0 / n[0], bc, bc)
+        cs = mx.cell_shape(g)
+        gs.append(g)
+        rho.append(cuda(np.exp(0.5 * rng.standard_normal(cs))))
+        beta0.append(cuda(np.exp(0.5 * rng.standard_normal(cs))))
+        sbar.append(cuda(rng.standard_normal(cs)))
+        us.append(W._periodic_faces(g, [torch.from_numpy(rng.standard_normal(g.face_shape(d))) for d in range(3)]))
+    opts = mx.default_opts(max_outer=2)
+    allow = (mx.MX_OK, mx.MX_ERR_NOCONV)
+    phi = [torch.zeros_like(r) for r in rho]
+    mx.mx_mac_project_batched(ctx, gs, *[[cuda(u[d].numpy()) for u in us] for d in range(3)], rho, beta0, sbar, phi,
+                              opts, allow=allow)
+    for b, g in enumerate(gs):
+        one = torch.zeros_like(rho[b])
+        mx.mx_mac_project(ctx, g, *[cuda(t.numpy()) for t in us[b]], rho[b], beta0[b], sbar[b], one, opts, allow=allow)
+        assert torch.equal(one, phi[b]), boxes[b]
