@@ -111,35 +111,51 @@ __device__ __forceinline__ double small_double(int a) {
 }
 
 // u += tab[K] a on the D-faces (an array of m2 planes of m01 = m0 x m1 faces, x
-// fastest), W0_PLANES planes of one column per thread: their loads are issued before
-// the first store.  Offsets fit 16 bits and K 29 (the table has at most 2^26
-// entries).  A thread per face of a plane: rows of n + 1 faces left a third of the
-// threads of 128-wide blocks without work.  HBM bound: 43 to 45 us per direction at
-// 256^3 (6.2 TB/s); 53 to 68 with a face at a time and converted offsets.
-constexpr int W0_PLANES = 4;
+// fastest).  A thread owns a face of the plane and four planes: two distances t from
+// the centre on either side of it, where K is the same, so a table entry serves two
+// faces (neighbouring faces' entries lie in different sectors, and the table's
+// traffic from L2 is what bounds the 512^3 box).  The four loads are issued before the first
+// store.  Offsets fit 16 bits and K 29 (the table has at most 2^26 entries).  A
+// thread per face of a plane: rows of n + 1 faces left a third of the threads of
+// 128-wide blocks without work.  The three directions with their table: 0.144 ms at
+// 256^3 (5.6 TB/s) and 1.10 at 512^3 (5.9 TB/s); 0.149 and 1.61 with four planes in a row,
+// 0.20 and 1.70 with a face at a time.
+constexpr int W0_PAIRS = 2;
+// the distances t0 .. t1 - 1 at which a box of m2 planes has one at c2 + t or, on the
+// other side, at c2 - t (D = 2) or c2 - 1 - t
+__host__ __device__ __forceinline__ int w0_first(int D, int m2, int c2) {
+    const int lo = c2 - m2 + (D == 2);
+    return lo > -c2 ? (lo > 0 ? lo : 0) : (-c2 > 0 ? -c2 : 0);
+}
+inline int w0_end(int D, int m2, int c2) { return std::max(m2 - c2, D == 2 ? c2 + 1 : c2); }
 template <int D>
 __global__ void __launch_bounds__(256) w0_faces_kernel(unsigned m0, unsigned m01, int m2, int c0, int c1, int c2,
                                                        const double *__restrict__ tab, double *__restrict__ u) {
     const unsigned p = blockIdx.x * 256u + threadIdx.x;
     if (p >= m01) return;
-    const int j = int(p / m0), i = int(p - unsigned(j) * m0), k0 = int(blockIdx.y) * W0_PLANES;
+    const int j = int(p / m0), i = int(p - unsigned(j) * m0);
+    const int t0 = w0_first(D, m2, c2) + int(blockIdx.y) * W0_PAIRS;
     // twice the offsets from the centre: even along D, odd along the others
     const int x = 2 * (i - c0) + (D != 0), y = 2 * (j - c1) + (D != 1);
-    const int Kxy = x * x + y * y, n = min(W0_PLANES, m2 - k0);
-    double *f = u + p + (long long)m01 * k0;
-    double v[W0_PLANES], w[W0_PLANES];
+    const int Kxy = x * x + y * y;
+    double v[2 * W0_PAIRS], w[W0_PAIRS];
+    int k[2 * W0_PAIRS];  // -1: no plane
 #pragma unroll
-    for (int q = 0; q < W0_PLANES; q++) {
-        if (q >= n) continue;
-        const int z = 2 * (k0 + q - c2) + (D != 2);
-        v[q] = f[(long long)m01 * q];
-        w[q] = __ldg(tab + ((Kxy + z * z) >> 2));  // K = 4 t + 2
+    for (int q = 0; q < W0_PAIRS; q++) {
+        const int t = t0 + q, up = c2 + t, dn = D == 2 ? c2 - t : c2 - 1 - t;
+        k[2 * q] = up >= 0 && up < m2 ? up : -1;
+        k[2 * q + 1] = dn >= 0 && dn < m2 && dn != up ? dn : -1;
+        const int z = 2 * t + (D != 2);
+        if (k[2 * q] >= 0 || k[2 * q + 1] >= 0) w[q] = __ldg(tab + ((Kxy + z * z) >> 2));  // K = 4 s + 2
+#pragma unroll
+        for (int s = 2 * q; s < 2 * q + 2; s++)
+            if (k[s] >= 0) v[s] = u[p + (long long)m01 * k[s]];
     }
 #pragma unroll
-    for (int q = 0; q < W0_PLANES; q++) {
-        if (q >= n) continue;
-        const int a = D == 0 ? i - c0 : (D == 1 ? j - c1 : k0 + q - c2);
-        f[(long long)m01 * q] = fma(w[q], small_double(a), v[q]);
+    for (int s = 0; s < 2 * W0_PAIRS; s++) {
+        if (k[s] < 0) continue;
+        const int a = D == 0 ? i - c0 : (D == 1 ? j - c1 : k[s] - c2);
+        u[p + (long long)m01 * k[s]] = fma(w[s >> 1], small_double(a), v[s]);
     }
 }
 
@@ -234,14 +250,15 @@ mx_status mx_add_w0_faces(mx_ctx *c, const mx_geom *geom, int spherical, const i
         return st;
     double *tab = (double *)c->split_tab;
     w0_table_kernel<<<(unsigned)((qmax + 256) / 256), 256, 0, c->stream>>>(qmax, geom->dx, nr, r_edge, w0, tab);
-    auto grid = [&](int m0, int m1, int m2) {
-        return dim3(unsigned(((long long)m0 * m1 + 255) / 256), (m2 + W0_PLANES - 1) / W0_PLANES);
+    auto grid = [&](int D, int m0, int m1, int m2) {
+        const int nt = w0_end(D, m2, corner[2]) - w0_first(D, m2, corner[2]);
+        return dim3(unsigned(((long long)m0 * m1 + 255) / 256), (nt + W0_PAIRS - 1) / W0_PAIRS);
     };
-    w0_faces_kernel<0><<<grid(n0 + 1, n1, n2), 256, 0, c->stream>>>(n0 + 1, (n0 + 1) * n1, n2, corner[0], corner[1],
+    w0_faces_kernel<0><<<grid(0, n0 + 1, n1, n2), 256, 0, c->stream>>>(n0 + 1, (n0 + 1) * n1, n2, corner[0], corner[1],
                                                                     corner[2], tab, ux);
-    w0_faces_kernel<1><<<grid(n0, n1 + 1, n2), 256, 0, c->stream>>>(n0, n0 * (n1 + 1), n2, corner[0], corner[1],
+    w0_faces_kernel<1><<<grid(1, n0, n1 + 1, n2), 256, 0, c->stream>>>(n0, n0 * (n1 + 1), n2, corner[0], corner[1],
                                                                     corner[2], tab, uy);
-    w0_faces_kernel<2><<<grid(n0, n1, n2 + 1), 256, 0, c->stream>>>(n0, n0 * n1, n2 + 1, corner[0], corner[1],
+    w0_faces_kernel<2><<<grid(2, n0, n1, n2 + 1), 256, 0, c->stream>>>(n0, n0 * n1, n2 + 1, corner[0], corner[1],
                                                                     corner[2], tab, uz);
     MX_CUDA(c, cudaGetLastError());
     return MX_OK;
