@@ -1,7 +1,7 @@
 // Cell-centred geometric multigrid kernels (MAC projection solve, Appendix A):
 // red-black Gauss-Seidel, residual + 8-cell-average restriction,
-// piecewise-constant prolongation, coefficient coarsening, a single-CTA
-// BiCGStab bottom solve, and the FP64 residual / update of the refinement loop.
+// piecewise-constant prolongation, coefficient coarsening, and the FP64 residual /
+// update of the refinement loop.
 // Templated on the V-cycle precision T (float for the mixed-precision path,
 // double for the plain FP64 path).
 #include "mx_rbgs.cuh"
