@@ -545,7 +545,7 @@ void k_resid_restrict(cudaStream_t s, const Level<T> &fine, const Level<T> &coar
             }
         }
         if constexpr (sizeof(T) == sizeof(float)) {
-            if (g.N >= RESTRICT_QUAD_MIN && resid_restrict_quad_ok(fine)) {
+            if (g.N >= RESTRICT_QUAD_MIN && g.n[0] >= 32 && resid_restrict_quad_ok(fine)) {
                 int zcf = 16;
                 auto grid = [&] { return resid_restrict_fine_grid(g, zcf, true); };
                 while (zcf > 2 && (long long)grid().x * grid().y * grid().z < 8 * 4 * 152) zcf >>= 1;
