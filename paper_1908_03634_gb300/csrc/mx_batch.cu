@@ -49,12 +49,14 @@ struct BatchPlan {
     // graph of the loop
     cudaGraphExec_t graph = nullptr;
     int g_nu1 = -1, g_nu2 = -1, g_bot = -1;
+    const double *g_part = nullptr;
     // side streams for the per-box setup and finish (small kernels of different
     // boxes overlap), each with its own slice of the reduction scratch
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> side_done;
     cudaEvent_t fork = nullptr;
     long long part_stride = 0;  // doubles per side stream in the partials
+    long long parts = 0;        // partial results of scratch a call needs
 };
 
 static void free_batch(BatchPlan *B) {
@@ -197,7 +199,8 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
     long long maxblk = 0;
     for (int b = 0; b < nbox; b++) maxblk = std::max<long long>(maxblk, std::max(stencil_blocks(g[b]), red_blocks(g[b].N)));
     B->part_stride = 3 * maxblk;
-    if ((*st = ensure_partials(c, std::max<long long>(std::max(parts, 152 * 8), NSIDE * maxblk)))) {
+    B->parts = std::max<long long>(std::max(parts, 152 * 8), NSIDE * maxblk);
+    if ((*st = ensure_partials(c, B->parts))) {
         free_batch(B);
         return nullptr;
     }
@@ -319,7 +322,8 @@ __global__ void batch_any_active_kernel(cudaGraphConditionalHandle h, const Solv
 }
 
 static mx_status batch_graph(mx_ctx *c, BatchPlan &B, const mx_opts &o) {
-    if (B.graph && B.g_nu1 == o.nu1 && B.g_nu2 == o.nu2 && B.g_bot == o.bottom_iters) return MX_OK;
+    if (B.graph && B.g_part == c->partials && B.g_nu1 == o.nu1 && B.g_nu2 == o.nu2 && B.g_bot == o.bottom_iters)
+        return MX_OK;
     if (B.graph) {
         cudaGraphExecDestroy(B.graph);
         B.graph = nullptr;
@@ -356,6 +360,7 @@ static mx_status batch_graph(mx_ctx *c, BatchPlan &B, const mx_opts &o) {
         B.graph = nullptr;
         return set_err(c, MX_ERR_CUDA, std::string("batched graph instantiate failed: ") + cudaGetErrorString(e));
     }
+    B.g_part = c->partials;
     B.g_nu1 = o.nu1;
     B.g_nu2 = o.nu2;
     B.g_bot = o.bottom_iters;
@@ -400,6 +405,7 @@ extern "C" mx_status mx_mac_project_batched(mx_ctx *c, int nbox, const mx_geom *
         if (!c->batch) return st;
     }
     BatchPlan &B = *c->batch;
+    if ((st = ensure_partials(c, B.parts))) return st;
     cudaStream_t s = c->stream;
     MX_CUDA(c, cudaEventRecord(c->ev0, s));
     for (int b = 0; b < nbox; b++) {

@@ -64,6 +64,7 @@ struct NodalPlan {
     // CUDA graph of the refinement loop, keyed by what it was captured with
     cudaGraphExec_t graph = nullptr;
     const void *graph_phi = nullptr;
+    const double *graph_part = nullptr;
     int graph_nu1 = -1, graph_nu2 = -1, graph_bot = -1, graph_tilez = -1, graph_smoother = -1;
     long long last_use = 0;
 };
@@ -2072,7 +2073,8 @@ static void free_nodal_plan(NodalPlan *p) {
 
 static NodalPlan *get_nodal_plan(mx_ctx *c, const NGeom &g, int prec, mx_status *st) {
     const dim3 tg = nd_df_tile_grid(g);
-    *st = ensure_partials(c, std::max<long long>(std::max(152 * 8, nd_col_blocks(g)), (long long)tg.x * tg.y * tg.z));
+    *st = ensure_partials(c, std::max<long long>(std::max(std::max(152 * 8, nd_col_blocks(g)), nd_node_blocks(g)),
+                                                 (long long)tg.x * tg.y * tg.z));
     if (*st) return nullptr;
     for (NodalPlan *p : c->nplans)
         if (p->prec == prec && same_ngeom(p->g, g)) {
@@ -2333,13 +2335,15 @@ extern "C" mx_status mx_nodal_project(mx_ctx *c, const mx_geom *geom, double *ux
         if (o.use_graph && !c->prof) {
             // the FP64 loop updates phi in place; the mixed loop never touches it
             const void *kphi = mixed ? nullptr : (const void *)phi;
-            if (!P->graph || P->graph_phi != kphi || P->graph_nu1 != o.nu1 || P->graph_nu2 != o.nu2 ||
+            if (!P->graph || P->graph_part != c->partials || P->graph_phi != kphi || P->graph_nu1 != o.nu1 ||
+                P->graph_nu2 != o.nu2 ||
                 P->graph_bot != o.bottom_iters || P->graph_tilez != o.tile_z || P->graph_smoother != o.smoother) {
                 if (P->graph) {
                     cudaGraphExecDestroy(P->graph);
                     P->graph = nullptr;
                 }
                 if ((st = capture_while_graph(c, &P->graph, [&](cudaStream_t cs) { step(cs, nullptr); }))) return st;
+                P->graph_part = c->partials;
                 P->graph_phi = kphi;
                 P->graph_nu1 = o.nu1;
                 P->graph_nu2 = o.nu2;

@@ -131,6 +131,9 @@ MacPlan *create_mac_plan(mx_ctx *c, const DGeom &g, int prec, mx_status *st) {
     return P;
 }
 
+// At least nblocks partial results of scratch.  Every kind of plan keeps its loop as a
+// graph that holds the scratch pointer, so each graph's key includes the pointer, and
+// a plan that is used again asks for its scratch again.
 mx_status ensure_partials(mx_ctx *c, long long nblocks) {
     if (nblocks <= c->max_partials) return MX_OK;
     cudaStreamSynchronize(c->stream);
@@ -142,11 +145,6 @@ mx_status ensure_partials(mx_ctx *c, long long nblocks) {
         return set_err(c, MX_ERR_OOM, "reduction scratch cudaMalloc failed");
     }
     c->max_partials = int(nblocks);
-    for (MacPlan *p : c->plans)  // graphs captured the old scratch pointer
-        if (p->graph) {
-            cudaGraphExecDestroy(p->graph);
-            p->graph = nullptr;
-        }
     return MX_OK;
 }
 
@@ -399,7 +397,7 @@ mx_status capture_while_graph(mx_ctx *c, cudaGraphExec_t *exec, const std::funct
 template <typename T>
 static mx_status run_loop_graph(mx_ctx *c, MacPlan &P, Hier<T> &H, double *phi, const mx_opts &o, int singular, int nb) {
     cudaStream_t s = c->stream;
-    if (!P.graph || P.graph_nu1 != o.nu1 || P.graph_nu2 != o.nu2 ||
+    if (!P.graph || P.graph_part != c->partials || P.graph_nu1 != o.nu1 || P.graph_nu2 != o.nu2 ||
         P.graph_bot != o.bottom_iters || P.graph_fused != o.fused || P.graph_tilez != o.tile_z ||
         P.graph_krylov != o.krylov) {
         if (P.graph) {
@@ -409,6 +407,7 @@ static mx_status run_loop_graph(mx_ctx *c, MacPlan &P, Hier<T> &H, double *phi, 
         mx_status st = capture_while_graph(
             c, &P.graph, [&](cudaStream_t cs) { ir_step(cs, c, P, H, phi, o, singular, nb, nullptr); });
         if (st) return st;
+        P.graph_part = c->partials;
         P.graph_nu1 = o.nu1;
         P.graph_nu2 = o.nu2;
         P.graph_bot = o.bottom_iters;

@@ -28,8 +28,10 @@ struct MacPlan {
     // FCG (mx_opts::krylov): two direction buffers and q = h^2 L p, allocated on first use
     float *kry_mem = nullptr;
     float *kp0 = nullptr, *kp1 = nullptr, *kq = nullptr;
-    // CUDA graph of the refinement loop, keyed by the options it was captured with
+    // CUDA graph of the refinement loop, keyed by the options and the
+    // reduction scratch it was captured with
     cudaGraphExec_t graph = nullptr;
+    const double *graph_part = nullptr;
     int graph_nu1 = -1, graph_nu2 = -1, graph_bot = -1, graph_fused = -1, graph_tilez = -1, graph_krylov = -1;
     long long last_use = 0;
 };
