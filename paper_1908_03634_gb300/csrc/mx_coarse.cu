@@ -63,7 +63,8 @@ __device__ __forceinline__ int fdiv(int x, FastDiv f) { return f.d == 1 ? x : in
 
 // One level of the coarse end.  Shared-memory offsets are in bytes and equal in
 // every CTA; the correction holds pp + 2 planes (a neighbour's plane first and
-// last), the right-hand side pp planes.
+// last), the right-hand side pp planes.  The bottom level, which only its own solve
+// visits, has no neighbours' planes: eoff lies a plane before its first cell.
 template <typename T>
 struct CoarseLevel {
     Level<T> L;
@@ -613,7 +614,8 @@ static bool plan_coarse(CoarseArgs<T> &A, const Level<T> *levs, int nl, int nc) 
     std::memset(&A, 0, sizeof(A));
     A.nl = nl;
     const int cap = CT * (nc > 1 ? CELLS_CLUSTER : CELLS_ALONE), B = sizeof(T);
-    long long off = 16, scratch = 0;  // bytes; the element at 0 stays 0
+    // bytes; the element at 0 stays 0 (the bottom alone has no use for it)
+    long long off = nl > 1 ? 16 : 0, scratch = 0;
     int used = 1;
     bool above_dist = true;
     for (int l = 0; l < nl; l++) {
@@ -639,9 +641,14 @@ static bool plan_coarse(CoarseArgs<T> &A, const Level<T> *levs, int nl, int nc) 
             if (g.N > COARSE_MAX_CELLS) return false;
             scratch = std::max(scratch, g.N > BOT_REGS * CT ? 6 * g.N : 2 * (g.N + 1));
         }
-        C.eoff = int(off);
-        off += (own + 2 * g.nxy) * B;
-        if (off > 65535) return false;  // neighbour offsets are 16 bits
+        if (l + 1 < nl) {
+            C.eoff = int(off);
+            off += (own + 2 * g.nxy) * B;
+            if (off > 65535) return false;  // neighbour offsets are 16 bits
+        } else {
+            C.eoff = int(off - g.nxy * B);
+            off += own * B;
+        }
     }
     for (int l = 0; l < nl; l++) {
         A.lev[l].foff = int(off);

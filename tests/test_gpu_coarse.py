@@ -80,3 +80,27 @@ def test_coarse_end_parity_and_batched_identity(mx, ctx, n, bc):
     mx.mx_mac_project_batched(ctx, [g], *[[cuda(t)] for t in u], [cuda(rho)], [cuda(beta0)], [cuda(sbar)], [phi],
                               mx.default_opts())
     assert np.array_equal(phi.cpu().numpy(), phis[1])
+
+
+@pytest.mark.parametrize("n,bc", [((64, 64, 1), (P, P, N)), ((128, 32, 1), (D, N, N)), ((1, 4096, 1), (N, D, D)),
+                                  ((5, 16, 32), (N, P, D)), ((13, 13, 15), (D, N, D))])
+def test_largest_bottoms(mx, ctx, n, bc):
+    """The largest bottoms the launch takes: 4096 cells in FP32 (one plane, one row), 2560
+    in FP64, whose vectors fill the shared memory.  Batched solves take no box without a
+    level that fits, so these calls fail where the layout leaves too little room.  The
+    residual is the one asked for, 1e-10 of max |f|, up to the rounding of the row's twelve
+    products (FP64; double-float coefficients in mixed solves), and the batched solve has the single one's bits."""
+    g, rho, beta0, sbar, u = problem(n, bc)
+    f, b = O.mac_rhs(g, u, beta0, sbar)[0], O.mac_coeffs(g, rho, beta0)
+    phis = []
+    for prec in (0, 1):
+        phi = torch.zeros(O.cell_shape(g), dtype=torch.float64, device=DEV)
+        mx.mx_mac_project(ctx, g, *[cuda(t) for t in u], cuda(rho), cuda(beta0), cuda(sbar), phi,
+                          mx.default_opts(prec=prec))
+        phis.append(phi.cpu().numpy())
+        rounding = 2.0 ** (-44 if prec else -48) * 12 * max(np.abs(x).max() for x in b) * np.abs(phis[-1]).max() / g.dx**2
+        assert np.abs(f - O.mac_apply(g, b, phis[-1])).max() <= 1e-10 * np.abs(f).max() + rounding
+    phi = torch.zeros(O.cell_shape(g), dtype=torch.float64, device=DEV)
+    mx.mx_mac_project_batched(ctx, [g], *[[cuda(t)] for t in u], [cuda(rho)], [cuda(beta0)], [cuda(sbar)], [phi],
+                              mx.default_opts())
+    assert np.array_equal(phi.cpu().numpy(), phis[1])
