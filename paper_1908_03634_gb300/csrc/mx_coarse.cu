@@ -285,7 +285,10 @@ __device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b)
 // the problem is singular; stops at relative residual 1e-4 or `iters`.  The
 // operator is preconditioned from the right with its diagonal (v = L D^-1 p, so
 // the residuals are those of L x = f): the stratified coefficients vary a hundredfold
-// over the bottom level.  Each of
+// over the bottom level.  What is solved is h^2 L x' = f' with f' = f 2^m of norm 1 to
+// 2 and x = x' h^2 / 2^m, so no sum or quotient depends on the unit of length or on
+// how far the outer iteration has come; in FP32 the sums of (L p)^2 would vanish with
+// cells of 1e8 units, and the quotients leave the fast division's range.  Each of
 // nthr threads (whole warps) holds up to B cells (cell t + q nthr): coefficients
 // and vectors stay in registers, and the vector the operator is applied to passes
 // through shared memory (element n holds 0 for faces without a neighbour).
@@ -299,9 +302,9 @@ __device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b)
 // agree bit for bit.
 template <typename T, int B>
 __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular,
-                                              T ih2, int nthr) {
+                                              T h2, int nthr) {
     const int n = int(L.g.N), nx = L.g.n[0], ny = L.g.n[1], nz = L.g.n[2], nxy = nx * ny;
-    T b[B][6], den[B], dinv[B], xv[B], r[B], r0[B], p[B], v[B];
+    T b[B][6], den[B], dinv[B], xv[B], r[B], r0[B] = {}, p[B], v[B];
     unsigned nb[B][3];
     if (threadIdx.x < 2) scr[threadIdx.x * (n + 1) + n] = T(0);
     T a[4] = {T(0), T(0), T(0), T(0)};
@@ -339,17 +342,22 @@ __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &
 #pragma unroll
     for (int q = 0; q < B; q++) {
         if (int(threadIdx.x) + q * nthr < n) r[q] -= mean;
-        r0[q] = r[q];
         a[0] = rfma(r[q], r[q], a[0]);
     }
     team.sum(a);
     rho1 = a[0];
+    T unit = T(1);
     if (rho1 > T(0)) {
+        unit = unit_scale(rho1);
+        rho1 = rho1 * unit * unit;
+#pragma unroll
+        for (int q = 0; q < B; q++) r0[q] = r[q] = r[q] * unit;
         tol2 = rho1 * T(1e-8);  // 1e-4 relative: ample for a multigrid bottom solve
 #pragma unroll 1
         for (int it = 0; it < iters; it++) {
-            if (rho1 == T(0) || omega == T(0)) break;
-            const T beta = sdiv(rho1 * alpha, rho * omega);
+            const T last = rho * omega;
+            if (rho1 == T(0) || fabs(last) < T(BREAKDOWN)) break;
+            const T beta = sdiv(rho1 * alpha, last);
             T w[B], y[B];
 #pragma unroll
             for (int q = 0; q < B; q++) w[q] = p[q] = rfma(beta, rfma(-omega, v[q], p[q]), r[q]);
@@ -367,7 +375,7 @@ __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &
                     const T s0 = rfma(b[q][0], e[nb[q][0] & 0xffffu], rmul(b[q][1], e[nb[q][0] >> 16]));
                     const T s1 = rfma(b[q][2], e[nb[q][1] & 0xffffu], rmul(b[q][3], e[nb[q][1] >> 16]));
                     const T s2 = rfma(b[q][4], e[nb[q][2] & 0xffffu], rmul(b[q][5], e[nb[q][2] >> 16]));
-                    y[q] = rmul(rfma(-den[q], rmul(w[q], dinv[q]), radd(radd(s0, s1), s2)), ih2);
+                    y[q] = rfma(-den[q], rmul(w[q], dinv[q]), radd(radd(s0, s1), s2));
                     a[0] = rfma(r0[q], y[q], a[0]);
                     a[1] = rfma(w[q], w[q], a[1]);
                     a[2] = rfma(y[q], y[q], a[2]);
@@ -375,7 +383,7 @@ __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &
                 }
                 team.sum(a);
                 if (h == 0) {
-                    stop = a[0] == T(0);
+                    stop = fabs(a[0]) < T(BREAKDOWN);
                     if (stop) break;
                     alpha = sdiv(rho1, a[0]);
 #pragma unroll
@@ -405,9 +413,11 @@ __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &
         team.sum(a);
         mean = a[0] * inv_n;
     }
+    const T back = h2 / unit;
 #pragma unroll
     for (int q = 0; q < B; q++)
-        if (int(threadIdx.x) + q * nthr < n) x[threadIdx.x + q * nthr] = xv[q] - (singular ? mean : T(0));
+        if (int(threadIdx.x) + q * nthr < n)
+            x[threadIdx.x + q * nthr] = rmul(xv[q] - (singular ? mean : T(0)), back);
 }
 
 // dot product accumulated in T (FP32 on the mixed path: the bottom solve only
@@ -431,15 +441,16 @@ __device__ T cta_dot(const T *a, const T *b, int n) {
     return out;
 }
 
+// y = h^2 L x
 template <typename T>
-__device__ void cta_apply(const Level<T> &L, const T *x, T *y, T ih2) {
+__device__ void cta_apply(const Level<T> &L, const T *x, T *y) {
     const DGeom &g = L.g;
     for (int c = threadIdx.x; c < g.N; c += CT) {
         const int i = c % g.n[0], r = c / g.n[0], j = r % g.n[1], k = r / g.n[1];
         T b[6], v[6];
         coefs32(L, i, j, k, c, b);
         nb_vals(g, x, i, j, k, c, v);
-        y[c] = flux_sum(b, v, x[c]) * ih2;
+        y[c] = flux_sum(b, v, x[c]);
     }
     __syncthreads();
 }
@@ -447,7 +458,7 @@ __device__ void cta_apply(const Level<T> &L, const T *x, T *y, T ih2) {
 // The same solve with its vectors in shared memory, for bottoms too large for
 // registers (levels that cannot be coarsened further).
 template <typename T>
-__device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular, T ih2) {
+__device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int iters, int singular, T h2) {
     const int n = int(L.g.N);
     T *r = scr, *r0 = scr + n, *p = scr + 2 * n, *v = scr + 3 * n, *sv = scr + 4 * n, *tv = scr + 5 * n;
     const T mean = singular ? cta_dot(f, (const T *)nullptr, n) / T(n) : T(0);
@@ -455,13 +466,16 @@ __device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int it
         const T b = f[q] - mean;
         x[q] = T(0);
         r[q] = b;
-        r0[q] = b;
         p[q] = T(0);
         v[q] = T(0);
     }
     __syncthreads();
-    const T bnorm2 = cta_dot(r, r, n);
+    T bnorm2 = cta_dot(r, r, n);
     if (!(bnorm2 > T(0))) return;
+    const T unit = unit_scale(bnorm2), back = h2 / unit;
+    bnorm2 = bnorm2 * unit * unit;
+    for (int q = threadIdx.x; q < n; q += CT) r0[q] = r[q] = r[q] * unit;
+    __syncthreads();
     const T tol2 = bnorm2 * T(1e-8);  // 1e-4 relative: ample for a multigrid bottom solve
     T rho = T(1), alpha = T(1), omega = T(1);
     for (int it = 0; it < iters; it++) {
@@ -470,7 +484,7 @@ __device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int it
         const T beta = (rho1 / rho) * (alpha / omega);
         for (int q = threadIdx.x; q < n; q += CT) p[q] = r[q] + beta * (p[q] - omega * v[q]);
         __syncthreads();
-        cta_apply(L, p, v, ih2);
+        cta_apply(L, p, v);
         const T r0v = cta_dot(r0, v, n);
         if (r0v == T(0)) break;
         alpha = rho1 / r0v;
@@ -482,7 +496,7 @@ __device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int it
             __syncthreads();
             break;
         }
-        cta_apply(L, sv, tv, ih2);
+        cta_apply(L, sv, tv);
         const T tt = cta_dot(tv, tv, n);
         const T ts = cta_dot(tv, sv, n);
         omega = tt > T(0) ? ts / tt : T(0);
@@ -495,11 +509,9 @@ __device__ void cta_bicgstab(const Level<T> &L, T *x, const T *f, T *scr, int it
         const T rr = cta_dot(r, r, n);
         if (rr <= tol2) break;
     }
-    if (singular) {
-        const T mx = cta_dot(x, (const T *)nullptr, n) / T(n);
-        for (int q = threadIdx.x; q < n; q += CT) x[q] -= mx;
-        __syncthreads();
-    }
+    const T mx = singular ? cta_dot(x, (const T *)nullptr, n) / T(n) : T(0);
+    for (int q = threadIdx.x; q < n; q += CT) x[q] = (x[q] - mx) * back;
+    __syncthreads();
 }
 
 // cells per thread, and threads, of a bottom solve in registers: the fewest warps that
@@ -511,16 +523,16 @@ __device__ __forceinline__ int bottom_threads(int n) {
 }
 
 template <typename T>
-__device__ void bottom_solve(TeamShared<T> &S, const Level<T> &L, T ih2, T *x, const T *f, T *scr, int iters, int singular) {
+__device__ void bottom_solve(TeamShared<T> &S, const Level<T> &L, T h2, T *x, const T *f, T *scr, int iters, int singular) {
     const int n = int(L.g.N);
     const int per = bottom_per(n), nthr = bottom_threads(n);
     if (!nthr) {
-        cta_bicgstab(L, x, f, scr, iters, singular, ih2);
+        cta_bicgstab(L, x, f, scr, iters, singular, h2);
         return;
     }
     if (int(threadIdx.x) < nthr) {
-        if (per == 1) team_bicgstab<T, 1>(S, L, x, f, scr, iters, singular, ih2, nthr);
-        else team_bicgstab<T, BOT_REGS>(S, L, x, f, scr, iters, singular, ih2, nthr);
+        if (per == 1) team_bicgstab<T, 1>(S, L, x, f, scr, iters, singular, h2, nthr);
+        else team_bicgstab<T, BOT_REGS>(S, L, x, f, scr, iters, singular, h2, nthr);
     }
     __syncthreads();
 }
@@ -543,7 +555,7 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &A, int rank) {
         if (step == nb) {
             const CoarseLevel<T> &C = A.lev[nb];
             if (rank == 0)
-                bottom_solve(bottom, C.L, C.ih2, &sm_at<T>(C.eoff + int(C.L.g.nxy) * B), &sm_at<T>(C.foff), &sm_at<T>(A.roff),
+                bottom_solve(bottom, C.L, C.h2, &sm_at<T>(C.eoff + int(C.L.g.nxy) * B), &sm_at<T>(C.foff), &sm_at<T>(A.roff),
                              A.bot_iters, A.singular);
             continue;
         }

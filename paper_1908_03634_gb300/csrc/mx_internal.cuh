@@ -94,6 +94,14 @@ __device__ __forceinline__ double nmax(double a, double b) {
     const long long ib = __double_as_longlong(b) & 0x7fffffffffffffffll;
     return __longlong_as_double(ia > ib ? ia : ib);
 }
+// 2^m with 4^-m the power of four at or below v > 0: scaled by it, a vector of squared
+// norm v has one in [1, 4), without rounding.
+__device__ __forceinline__ float unit_scale(float v) {
+    return __int_as_float((127 - (((__float_as_int(v) >> 23) - 127) >> 1)) << 23);
+}
+__device__ __forceinline__ double unit_scale(double v) {
+    return __hiloint2double((1023 - (((__double2hiint(v) >> 20) - 1023) >> 1)) << 20, 0);
+}
 __device__ __forceinline__ float nmaxf(float a, float b) {
     float r;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));

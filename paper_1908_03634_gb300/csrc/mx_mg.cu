@@ -665,21 +665,23 @@ __device__ T bot_dot(const T *a, const T *b, int n) {
     return T(res);
 }
 
+// y = h^2 L x
 template <typename T>
-__device__ void bot_apply(const Level<T> &L, const T *x, T *y, T ih2) {
+__device__ void bot_apply(const Level<T> &L, const T *x, T *y) {
     const DGeom &g = L.g;
     for (int c = threadIdx.x; c < g.N; c += BOT_THREADS) {
         const int i = c % g.n[0], j = (c / g.n[0]) % g.n[1], k = c / (g.n[0] * g.n[1]);
         T b[6], v[6];
         face_coefs(L, i, j, k, c, b);
         nb_vals(g, x, i, j, k, c, v);
-        y[c] = flux_sum(b, v, x[c]) * ih2;
+        y[c] = flux_sum(b, v, x[c]);
     }
     __syncthreads();
 }
 
+// As in the coarse end's bottom solves, h^2 L x' = f' with f' = f 2^m of norm 1 to 2.
 template <typename T>
-__global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr, int iters, int singular, T ih2) {
+__global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr, int iters, int singular, T h2) {
     pdl_trigger();
     pdl_wait();
     const int n = int(L.g.N);
@@ -701,14 +703,16 @@ __global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr,
         const T b = L.f[q] - mean;
         bvec[q] = b;
         x[q] = T(0);
-        r[q] = b;
-        r0[q] = b;
         p[q] = T(0);
         v[q] = T(0);
     }
     __syncthreads();
-    const T bnorm2 = bot_dot(bvec, bvec, n);
+    T bnorm2 = bot_dot(bvec, bvec, n);
     if (!(bnorm2 > T(0))) return;
+    const T unit = unit_scale(bnorm2), back = h2 / unit;
+    bnorm2 = bnorm2 * unit * unit;
+    for (int q = threadIdx.x; q < n; q += BOT_THREADS) r0[q] = r[q] = bvec[q] * unit;
+    __syncthreads();
     const T tol2 = bnorm2 * T(1e-8);  // 1e-4 relative: ample for a multigrid bottom solve
     T rho = T(1), alpha = T(1), omega = T(1);
     for (int it = 0; it < iters; it++) {
@@ -717,7 +721,7 @@ __global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr,
         const T beta = (rho1 / rho) * (alpha / omega);
         for (int q = threadIdx.x; q < n; q += BOT_THREADS) p[q] = r[q] + beta * (p[q] - omega * v[q]);
         __syncthreads();
-        bot_apply(L, p, v, ih2);
+        bot_apply(L, p, v);
         const T r0v = bot_dot(r0, v, n);
         if (r0v == T(0)) break;
         alpha = rho1 / r0v;
@@ -729,7 +733,7 @@ __global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr,
             __syncthreads();
             break;
         }
-        bot_apply(L, sv, tv, ih2);
+        bot_apply(L, sv, tv);
         const T tt = bot_dot(tv, tv, n);
         const T ts = bot_dot(tv, sv, n);
         omega = tt > T(0) ? ts / tt : T(0);
@@ -742,6 +746,7 @@ __global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr,
         const T rr = bot_dot(r, r, n);
         if (rr <= tol2) break;
     }
+    T mx = T(0);
     if (singular) {
         double s = 0.0;
         for (int q = threadIdx.x; q < n; q += BOT_THREADS) s += double(x[q]);
@@ -750,15 +755,15 @@ __global__ void __launch_bounds__(BOT_THREADS) bottom_kernel(Level<T> L, T *scr,
         __shared__ double sm2;
         if (threadIdx.x == 0) sm2 = s / n;
         __syncthreads();
-        const T mx = T(sm2);
-        for (int q = threadIdx.x; q < n; q += BOT_THREADS) x[q] -= mx;
+        mx = T(sm2);
     }
+    for (int q = threadIdx.x; q < n; q += BOT_THREADS) x[q] = (x[q] - mx) * back;
 }
 
 template <typename T>
 void k_bottom(cudaStream_t s, const Level<T> &L, T *scratch, int iters, int singular) {
     const double h = L.g.h;
-    launch_pdl(bottom_kernel<T>, dim3(1), dim3(BOT_THREADS), 0, s, L, scratch, iters, singular, T(1.0 / (h * h)));
+    launch_pdl(bottom_kernel<T>, dim3(1), dim3(BOT_THREADS), 0, s, L, scratch, iters, singular, T(h * h));
 }
 
 // ------------------------------------------------------------------------------

@@ -501,9 +501,9 @@ static int nd_xfer_zc(const NGeom &g) {
 }
 
 
-// y = L x
+// y = L x h^2 / h2 (h2 = h^2: the operator; 1: the operator in units of the cell width)
 template <typename T>
-__device__ void nd_apply_one(const NLevel<T> &L, const T *x, T *y, long long q) {
+__device__ void nd_apply_one(const NLevel<T> &L, const T *x, T *y, long long q, T h2) {
     const NGeom &g = L.g;
     int a, b, c;
     node_of(g, q, a, b, c);
@@ -514,13 +514,13 @@ __device__ void nd_apply_one(const NLevel<T> &L, const T *x, T *y, long long q) 
         if (m >= 0) num += coef * x[m];
         den += coef;
     });
-    y[q] = (num - den * x[q]) / (T(12) * T(node_w(g, a, b, c)) * T(g.h * g.h));
+    y[q] = (num - den * x[q]) / (T(12) * T(node_w(g, a, b, c)) * h2);
 }
 
 template <typename T>
 __global__ void nd_apply_kernel(NLevel<T> L, const T *x, T *y) {
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < L.g.M; q += (long long)gridDim.x * blockDim.x)
-        nd_apply_one(L, x, y, q);
+        nd_apply_one(L, x, y, q, T(L.g.h * L.g.h));
 }
 
 // BiCGStab on the coarsest nodal level (one CTA).  The nodal operator is
@@ -569,6 +569,7 @@ __device__ void nd_wmean0(const NGeom &g, T *x) {
 // holds 0), the two applications of an iteration through one rolled body with one
 // reduction each, right-preconditioned with the diagonal (the cell-centred bottom
 // solve has the same form).
+// As there, what is solved is h^2 L x' = f' with f' = f 2^m of norm 1 to 2.
 // The cost is instruction fetch and the latency of the sums: 240 nodes took 318 us
 // per V-cycle when every product re-read the 8 cells and every sum was its own
 // block-wide reduction.
@@ -617,7 +618,7 @@ __device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &
             m++;
         }
         w = node_w(g, a, b, c);
-        inv = T(1) / (T(12) * T(w) * T(g.h * g.h));
+        inv = T(1) / (T(12) * T(w));
         dinv = den != T(0) ? T(1) / (den * inv) : T(0);
         r = L.f[q];
     }
@@ -625,18 +626,22 @@ __device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &
     team.sum(a);
     const float wsum = a[1];
     if (q < n) r -= T(a[0] / wsum);  // compatibility (all nodal problems here are singular)
-    const T r0 = r;
     T x = T(0), p = T(0), v = T(0);
     a[0] = w * float(r) * float(r);
     a[1] = a[2] = a[3] = 0.f;
     team.sum(a);
-    float rho1 = a[0], rho = 1.f, alpha = 1.f, omega = 1.f;
+    float rho1 = a[0], rho = 1.f, alpha = 1.f, omega = 1.f, unit = 1.f;
     if (rho1 > 0.f) {
+        unit = unit_scale(rho1);
+        rho1 = rho1 * unit * unit;
+        r *= T(unit);
+        const T r0 = r;
         const float tol2 = rho1 * 1e-8f;
 #pragma unroll 1
         for (int it = 0; it < iters; it++) {
-            if (rho1 == 0.f || omega == 0.f) break;
-            p = r + T(sdiv(rho1 * alpha, rho * omega)) * (p - T(omega) * v);
+            const float last = rho * omega;
+            if (rho1 == 0.f || fabsf(last) < float(BREAKDOWN)) break;
+            p = r + T(sdiv(rho1 * alpha, last)) * (p - T(omega) * v);
             T u = p, y = T(0);
             bool stop = false;
 #pragma unroll 1
@@ -659,7 +664,7 @@ __device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &
                 a[3] = wy * fu;
                 team.sum(a);
                 if (h == 0) {
-                    stop = a[0] == 0.f;
+                    stop = fabsf(a[0]) < float(BREAKDOWN);
                     if (stop) break;
                     alpha = sdiv(rho1, a[0]);
                     v = y;
@@ -679,7 +684,7 @@ __device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &
     a[0] = w * float(x);
     a[1] = a[2] = a[3] = 0.f;
     team.sum(a);
-    if (q < n) L.e[q] = x - T(a[0] / wsum);
+    if (q < n) L.e[q] = (x - T(a[0] / wsum)) * (T(g.h * g.h) / T(unit));
 }
 
 template <typename T>
@@ -702,13 +707,16 @@ __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int
     nd_wmean0(g, r);  // compatibility (all nodal problems here are singular)
     for (int q = threadIdx.x; q < n; q += NBT) {
         x[q] = T(0);
-        r0[q] = r[q];
         p[q] = T(0);
         v[q] = T(0);
     }
     __syncthreads();
-    const T bnorm2 = nd_wdot(g, r, r, 1);
+    T bnorm2 = nd_wdot(g, r, r, 1);
     if (!(bnorm2 > T(0))) return;
+    const T unit = unit_scale(bnorm2), back = T(g.h * g.h) / unit;
+    bnorm2 = bnorm2 * unit * unit;
+    for (int q = threadIdx.x; q < n; q += NBT) r0[q] = r[q] = r[q] * unit;
+    __syncthreads();
     const T tol2 = bnorm2 * T(1e-8);
     T rho = T(1), alpha = T(1), omega = T(1);
     for (int it = 0; it < iters; it++) {
@@ -717,7 +725,7 @@ __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int
         const T beta = (rho1 / rho) * (alpha / omega);
         for (int q = threadIdx.x; q < n; q += NBT) p[q] = r[q] + beta * (p[q] - omega * v[q]);
         __syncthreads();
-        for (int q = threadIdx.x; q < n; q += NBT) nd_apply_one(L, p, v, q);
+        for (int q = threadIdx.x; q < n; q += NBT) nd_apply_one(L, p, v, q, T(1));
         __syncthreads();
         const T r0v = nd_wdot(g, r0, v, 1);
         if (r0v == T(0)) break;
@@ -729,7 +737,7 @@ __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int
             __syncthreads();
             break;
         }
-        for (int q = threadIdx.x; q < n; q += NBT) nd_apply_one(L, sv, tv, q);
+        for (int q = threadIdx.x; q < n; q += NBT) nd_apply_one(L, sv, tv, q, T(1));
         __syncthreads();
         const T tt = nd_wdot(g, tv, tv, 1), ts = nd_wdot(g, tv, sv, 1);
         omega = tt > T(0) ? ts / tt : T(0);
@@ -742,6 +750,7 @@ __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int
         if (nd_wdot(g, r, r, 1) <= tol2) break;
     }
     nd_wmean0(g, x);
+    for (int q = threadIdx.x; q < n; q += NBT) x[q] *= back;
 }
 
 // ---- column-marching kernels ------------------------------------------------------------

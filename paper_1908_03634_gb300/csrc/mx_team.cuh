@@ -106,6 +106,10 @@ struct TeamSum {
     }
 };
 
+// Denominators of a bottom solve on vectors of norm 1 to 2 below this count as a
+// breakdown; it keeps the divisions by them in the fast form's range.
+#define BREAKDOWN 1e-30
+
 // The bottom solves' scalar divisions: they set step lengths, so the fast forms
 // (a division subroutine's instructions would cost more than its arithmetic).
 __device__ __forceinline__ float sdiv(float a, float b) { return __fdividef(a, b); }
