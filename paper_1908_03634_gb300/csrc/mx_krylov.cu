@@ -18,9 +18,15 @@
 // is the refinement step.  The directions and q are FP32: they set the step
 // sizes only, never the residual that decides convergence.
 //
+// The directions are stored as P = c p and Q = c q with c the power of two next to
+// 1/h^2: e is about h^2 rhat, and in FP32 the sums of its squares would leave the
+// type's range on cells of 1e8 units or of 1e-7.  Neither beta nor t P depends on c.
+//
 // Storage: two direction buffers alternating with the V-cycle count (a tile's
 // halo is staged from the previous direction while other tiles write the new
 // one) and q, written in place (only the next iteration's dot product reads it).
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "mx_krylov.cuh"
@@ -38,10 +44,10 @@ __device__ __forceinline__ int kmap(int u, int n, bool per) {
     return u < 0 ? u + n : u - n;
 }
 
-// per-block partials (0, e . q_prev, 0); nothing is read on a restart
+// per-block partials (0, c e . Q_prev, 0); nothing is read on a restart
 template <bool VEC>
 __global__ void __launch_bounds__(256) kry_dot_kernel(const float *__restrict__ e, const float *__restrict__ q,
-                                                      long long n, const SolveState *st, double *part) {
+                                                      long long n, float c, const SolveState *st, double *part) {
     float s = 0.f;
     if (!st->kry_restart) {
         const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -53,14 +59,14 @@ __global__ void __launch_bounds__(256) kry_dot_kernel(const float *__restrict__ 
             const float4 *__restrict__ q4 = reinterpret_cast<const float4 *>(q);
             for (long long i = t0; i < n4; i += stride) {
                 const float4 a = e4[i], b = q4[i];
-                s = fmaf(a.x, b.x, s);
-                s = fmaf(a.y, b.y, s);
-                s = fmaf(a.z, b.z, s);
-                s = fmaf(a.w, b.w, s);
+                s = fmaf(c * a.x, b.x, s);
+                s = fmaf(c * a.y, b.y, s);
+                s = fmaf(c * a.z, b.z, s);
+                s = fmaf(c * a.w, b.w, s);
             }
             done = n4 << 2;
         }
-        for (long long i = done + t0; i < n; i += stride) s = fmaf(e[i], q[i], s);
+        for (long long i = done + t0; i < n; i += stride) s = fmaf(c * e[i], q[i], s);
     }
     float z0 = 0.f, z2 = 0.f;
     block_red3f(z0, s, z2);
@@ -85,11 +91,11 @@ __global__ void kry_beta_kernel(const double *part, int nb, SolveState *st) {
     }
 }
 
-// p = e + beta p_prev staged with a one-cell halo (zero outside the box on
+// P = c e + beta P_prev staged with a one-cell halo (zero outside the box on
 // non-periodic axes, as the stored boundary coefficients expect), written to
-// the buffer of this iteration; q = h^2 L p; partials (0, p . q, p . rhat).
+// the buffer of this iteration; Q = h^2 L P; partials (0, P . Q, P . rhat).
 __global__ void __launch_bounds__(K_THREADS) kry_dir_kernel(Level<float> L, const float *__restrict__ e,
-                                                            float *p0, float *p1, float *__restrict__ q,
+                                                            float *p0, float *p1, float *__restrict__ q, float ce,
                                                             const SolveState *st, double *part) {
     __shared__ float sp[KHZ][KHY][KHX];
     const DGeom &g = L.g;
@@ -108,7 +114,7 @@ __global__ void __launch_bounds__(K_THREADS) kry_dir_kernel(Level<float> L, cons
         float v = 0.f;
         if (lx >= 0 && ly >= 0 && lz >= 0) {
             const long long c = lx + (long long)nx * (ly + (long long)ny * lz);
-            v = e[c];
+            v = ce * e[c];
             if (!restart) v = fmaf(beta, po[c], v);
         }
         sp[az][ay][ax] = v;
@@ -149,7 +155,7 @@ __global__ void __launch_bounds__(K_THREADS) kry_dir_kernel(Level<float> L, cons
     }
 }
 
-// the line-search step t into the update step of the residual kernel; a
+// the line-search step t / c into the update step of the residual kernel; a
 // direction that is not a descent direction of the energy (p . q >= 0, or a
 // non-finite sum) takes t = 0 and restarts from p = e
 __global__ void kry_step_kernel(const double *part, int nb, SolveState *st, double h2) {
@@ -176,11 +182,18 @@ __global__ void kry_step_kernel(const double *part, int nb, SolveState *st, doub
 
 }  // namespace
 
-void k_kry_dot(cudaStream_t s, long long n, const float *e, const float *q, SolveState *st, double *partials) {
+// the power of two at or next above 1/h^2, within FP32's normal range
+static float dir_scale(const DGeom &g) {
+    return std::ldexp(1.f, std::min(126, std::max(-126, -std::ilogb(g.h * g.h))));
+}
+
+void k_kry_dot(cudaStream_t s, const DGeom &g, const float *e, const float *q, SolveState *st, double *partials) {
+    const long long n = g.N;
+    const float c = dir_scale(g);
     const int nb = red_blocks(n);
     const bool vec = ((reinterpret_cast<uintptr_t>(e) | reinterpret_cast<uintptr_t>(q)) & 15) == 0;
-    if (vec) kry_dot_kernel<true><<<nb, 256, 0, s>>>(e, q, n, st, partials);
-    else kry_dot_kernel<false><<<nb, 256, 0, s>>>(e, q, n, st, partials);
+    if (vec) kry_dot_kernel<true><<<nb, 256, 0, s>>>(e, q, n, c, st, partials);
+    else kry_dot_kernel<false><<<nb, 256, 0, s>>>(e, q, n, c, st, partials);
     kry_beta_kernel<<<1, 1024, 0, s>>>(partials, nb, st);
 }
 
@@ -188,7 +201,7 @@ void k_kry_dir(cudaStream_t s, const Level<float> &L0, const float *e, float *p0
                SolveState *st, double *partials) {
     const DGeom &g = L0.g;
     const dim3 grid((g.n[0] + KX - 1) / KX, (g.n[1] + KY - 1) / KY, (g.n[2] + KZ - 1) / KZ);
-    kry_dir_kernel<<<grid, K_THREADS, 0, s>>>(L0, e, p0, p1, q, st, partials);
+    kry_dir_kernel<<<grid, K_THREADS, 0, s>>>(L0, e, p0, p1, q, dir_scale(g), st, partials);
     kry_step_kernel<<<1, 1024, 0, s>>>(partials, int(grid.x * grid.y * grid.z), st, g.h * g.h);
 }
 

@@ -303,7 +303,7 @@ static void fcg_body(cudaStream_t s, mx_ctx *c, MacPlan &P, Hier<float> &H, cons
     vcycle(s, H, o.nu1, o.nu2, o.bottom_iters, singular, pc, o.fused, o.tile_z ? o.tile_z : 8);
     Level<float> &L0 = H.lev[0];
     prof_begin(pc, s, MX_PH_UPDATE);
-    k_kry_dot(s, P.g.N, L0.e, P.kq, c->state, c->partials);
+    k_kry_dot(s, P.g, L0.e, P.kq, c->state, c->partials);
     k_kry_dir(s, L0, L0.e, P.kp0, P.kp1, P.kq, c->state, c->partials);
     prof_end(pc, s, MX_PH_UPDATE, 4);
     prof_begin(pc, s, MX_PH_RESID64);

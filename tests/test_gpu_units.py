@@ -74,6 +74,11 @@ def test_mac_in_other_units(mx, ctx, n, bc, kw, s):
 
 
 @pytest.mark.parametrize("s", SCALES)
+def test_mac_fcg_in_other_units(mx, ctx, s):
+    test_mac_in_other_units(mx, ctx, (20, 24, 28), (P, P, N), {"krylov": 1}, s)
+
+
+@pytest.mark.parametrize("s", SCALES)
 @pytest.mark.parametrize("n,bc,kw", [((24, 20, 28), (P, P, N), {}), ((12, 20, 28), (N, N, N), {"smoother": 1}),
                                      ((18, 14, 22), (N, N, N), {})])
 def test_nodal_in_other_units(mx, ctx, n, bc, kw, s):
