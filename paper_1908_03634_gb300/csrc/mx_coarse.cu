@@ -279,8 +279,6 @@ __device__ __forceinline__ void visit(const CoarseArgs<T> &A, int l, int rank, b
     }
 }
 
-__device__ __forceinline__ double sdiv(double a, double b) { return a * rcp64(b); }
-
 // BiCGStab on L x = f (x starts at 0), projected onto mean-free vectors when
 // the problem is singular; stops at relative residual 1e-4 or `iters`.  The
 // operator is preconditioned from the right with its diagonal (v = L D^-1 p, so

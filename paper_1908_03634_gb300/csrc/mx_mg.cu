@@ -42,9 +42,9 @@ void k_coarsen_coeffs(cudaStream_t s, const Level<T> &fine, const Level<T> &coar
     coarsen_coeffs_kernel<T><<<unsigned((n + 255) / 256), 256, 0, s>>>(fine, coarse);
 }
 
-// The FP64 smoother's divisions, once per solve: 23 FP64 operations per update
-// with the division inside, 8 with the stored reciprocal (the FP64 pipe bounds the
-// colour pass).
+// The FP64 smoother's divisions, once per solve and correctly rounded: 23 FP64
+// operations per update with the division inside, 8 with the stored reciprocal (the
+// FP64 pipe bounds the colour pass).
 __global__ void inverse_diag_kernel(Level<double> L) {
     const DGeom &g = L.g;
     const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;

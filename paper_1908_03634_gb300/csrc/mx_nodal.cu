@@ -630,18 +630,19 @@ __device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &
     a[0] = w * float(r) * float(r);
     a[1] = a[2] = a[3] = 0.f;
     team.sum(a);
-    float rho1 = a[0], rho = 1.f, alpha = 1.f, omega = 1.f, unit = 1.f;
-    if (rho1 > 0.f) {
+    // the sums are FP32, the scalars of an FP64 solve FP64
+    T rho1 = T(a[0]), rho = T(1), alpha = T(1), omega = T(1), unit = T(1);
+    if (rho1 > T(0)) {
         unit = unit_scale(rho1);
         rho1 = rho1 * unit * unit;
-        r *= T(unit);
+        r *= unit;
         const T r0 = r;
-        const float tol2 = rho1 * 1e-8f;
+        const T tol2 = rho1 * T(1e-8);
 #pragma unroll 1
         for (int it = 0; it < iters; it++) {
-            const float last = rho * omega;
-            if (rho1 == 0.f || fabsf(last) < float(BREAKDOWN)) break;
-            p = r + T(sdiv(rho1 * alpha, last)) * (p - T(omega) * v);
+            const T last = rho * omega;
+            if (rho1 == T(0) || fabs(last) < T(BREAKDOWN)) break;
+            p = r + sdiv(rho1 * alpha, last) * (p - omega * v);
             T u = p, y = T(0);
             bool stop = false;
 #pragma unroll 1
@@ -666,25 +667,25 @@ __device__ __forceinline__ void nd_team_bicgstab(NdTeam<T> &S, const NLevel<T> &
                 if (h == 0) {
                     stop = fabsf(a[0]) < float(BREAKDOWN);
                     if (stop) break;
-                    alpha = sdiv(rho1, a[0]);
+                    alpha = sdiv(rho1, T(a[0]));
                     v = y;
-                    u = r - T(alpha) * y;
+                    u = r - alpha * y;
                 }
             }
             if (stop) break;
-            const bool small = a[1] <= tol2;
-            omega = !small && a[2] > 0.f ? sdiv(a[3], a[2]) : 0.f;
-            x += (T(alpha) * p + T(omega) * u) * dinv;
-            r = u - T(omega) * y;
-            if (small || a[1] - omega * (2.f * a[3] - omega * a[2]) <= tol2) break;
+            const bool small = T(a[1]) <= tol2;
+            omega = !small && a[2] > 0.f ? sdiv(T(a[3]), T(a[2])) : T(0);
+            x += (alpha * p + omega * u) * dinv;
+            r = u - omega * y;
+            if (small || T(a[1]) - omega * (T(2) * T(a[3]) - omega * T(a[2])) <= tol2) break;
             rho = rho1;
-            rho1 = -omega * a[0];
+            rho1 = -omega * T(a[0]);
         }
     }
     a[0] = w * float(x);
     a[1] = a[2] = a[3] = 0.f;
     team.sum(a);
-    if (q < n) L.e[q] = (x - T(a[0] / wsum)) * (T(g.h * g.h) / T(unit));
+    if (q < n) L.e[q] = (x - T(a[0] / wsum)) * (T(g.h * g.h) / unit);
 }
 
 template <typename T>

@@ -12,7 +12,7 @@ enum { RB_PLAIN = 0, RB_ZERO = 1, RB_PROLONG = 2 };
 // bit for bit whatever FMA contractions the compiler would choose in each.
 // FP32 multiplies with the hardware's approximate reciprocal of the diagonal (1
 // ulp; subnormal sums, far below any face-coefficient sum here, count as 0), FP64
-// with a reciprocal within 2 ulp.  The smoother only sets the V-cycle's
+// with a correctly rounded one.  The smoother only sets the V-cycle's
 // contraction, the refinement loop the accuracy.
 __device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
@@ -25,7 +25,7 @@ __device__ __forceinline__ float rinv(float a) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
-__device__ __forceinline__ double rinv(double a) { return rcp64(a); }
+__device__ __forceinline__ double rinv(double a) { return __drcp_rn(a); }
 
 // 1 / sum_f b_f of a cell's row
 template <typename T>

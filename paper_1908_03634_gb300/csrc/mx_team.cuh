@@ -110,6 +110,8 @@ struct TeamSum {
 // breakdown; it keeps the divisions by them in the fast form's range.
 #define BREAKDOWN 1e-30
 
-// The bottom solves' scalar divisions: they set step lengths, so the fast forms
-// (a division subroutine's instructions would cost more than its arithmetic).
+// The bottom solves' scalar divisions: they set step lengths, so FP32 takes the fast
+// form (a division subroutine's instructions would cost more than its arithmetic);
+// FP64 solves divide in FP64.
 __device__ __forceinline__ float sdiv(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double sdiv(double a, double b) { return a / b; }

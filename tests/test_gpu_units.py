@@ -74,6 +74,12 @@ def test_mac_in_other_units(mx, ctx, n, bc, kw, s):
 
 
 @pytest.mark.parametrize("s", SCALES)
+@pytest.mark.parametrize("n,bc", [((20, 24, 28), (P, P, N)), ((22, 26, 18), (N, D, N)), ((13, 13, 13), (D, N, N))])
+def test_mac_fp64_in_other_units(mx, ctx, n, bc, s):
+    test_mac_in_other_units(mx, ctx, n, bc, {"prec": 0}, s)
+
+
+@pytest.mark.parametrize("s", SCALES)
 def test_mac_fcg_in_other_units(mx, ctx, s):
     test_mac_in_other_units(mx, ctx, (20, 24, 28), (P, P, N), {"krylov": 1}, s)
 
@@ -87,3 +93,9 @@ def test_nodal_in_other_units(mx, ctx, n, bc, kw, s):
     assert one["status"] == 0 and one["rel_resid"] <= 1e-10
     assert (info["status"], info["vcycles"]) == (0, one["vcycles"])
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("s", SCALES)
+@pytest.mark.parametrize("n,bc", [((24, 20, 28), (P, P, N)), ((18, 14, 22), (N, N, N))])
+def test_nodal_fp64_in_other_units(mx, ctx, n, bc, s):
+    test_nodal_in_other_units(mx, ctx, n, bc, {"prec": 0}, s)
