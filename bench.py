@@ -185,8 +185,8 @@ def launches_per_solve(g, o, vcycles, graph, krylov=0, sweep_cells=None, coarse_
     remove).  FCG (krylov = 1) adds 4 per iteration: the dot product, its
     finalize, the direction/stencil pass and the step finalize.  Checked against
     the ncu launch lists of the planar 256^3 solve.  sweep_cells: levels of at
-    least so many cells run single-pass sweeps without o.fused; coarse_cells: the
-    largest level of the coarse end."""
+    least so many cells run single-pass sweeps with o.fused = 0 (1: from 2^18 cells, 2:
+    none does); coarse_cells: the largest level of the coarse end."""
     dims = [list(g.n)]
     while all(d % 2 == 0 and d >= 4 for d in dims[-1]):
         dims.append([d // 2 for d in dims[-1]])
@@ -195,7 +195,7 @@ def launches_per_solve(g, o, vcycles, graph, krylov=0, sweep_cells=None, coarse_
     ldown = next((l for l in range(nlev) if ncell[l] <= coarse_cells), nlev - 1)
     per_iter = 1 + 2 + (1 if graph else 0) + (4 if krylov else 0)
     for l in range(ldown):
-        least = (1 << 18) if o.fused else sweep_cells
+        least = None if o.fused == 2 else (1 << 18) if o.fused else sweep_cells
         fused = least and ncell[l] >= least and dims[l][0] % 4 == 0 and dims[l][0] >= 32
         per_iter += (o.nu1 + 1 + o.nu2) if fused else (2 * o.nu1 + 1 + 1 + 2 * o.nu2)
     setup = 1 + 1 + (nlev - 1) + 4 + 2
@@ -368,7 +368,7 @@ def run_mx(args):
     sm_ms, sm_n = trace["smooth_fine"]
     per_launch_ms = sm_ms / max(sm_n, 1)
     # the tuned smoother: two colour passes (12 B/cell each) or single-pass sweeps (24 B/cell)
-    fused0 = ncell >= ((1 << 18) if tuned.fused else SWEEP_CELLS) and g.n[0] % 4 == 0
+    fused0 = tuned.fused != 2 and ncell >= ((1 << 18) if tuned.fused else SWEEP_CELLS) and g.n[0] % 4 == 0
     sweep_bytes = 2 * bpc["smooth_fine"] if fused0 else bpc["smooth_fine"]
     achieved = sweep_bytes * ncell / (per_launch_ms * 1e-3) / 1e9
     r_ms, r_n = trace["resid64"]

@@ -90,7 +90,8 @@ typedef struct {
                               fused on load, or two colour kernels (bit-identical results).
                               0 (default): sweeps on levels that outgrow the L2 cache;
                               1: on every level of 2^18 cells or more that allows them
-                              (n[0] a multiple of 4, at least 32) */
+                              (n[0] a multiple of 4, at least 32);
+                              2: colour kernels on every level */
     int tile_z;            /* cells per thread along z in the stencil kernels' tiles (the
                               largest z-chunk; smaller levels use fewer): 0 = default
                               (8 MAC, 16 nodal), else 1, 2, 4, 8 or 16; results do not

@@ -48,7 +48,7 @@ struct BatchPlan {
     size_t coarse_smem = 0;
     // graph of the loop
     cudaGraphExec_t graph = nullptr;
-    int g_nu1 = -1, g_nu2 = -1, g_bot = -1;
+    int g_nu1 = -1, g_nu2 = -1, g_bot = -1, g_fused = -1;
     const double *g_part = nullptr;
     // side streams for the per-box setup and finish (small kernels of different
     // boxes overlap), each with its own slice of the reduction scratch
@@ -131,7 +131,7 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
                 cells += gl.back().N;
                 sweeps = sweeps && rbgs_fused_ok(gl.back());
             }
-        if (sweeps && cells >= SWEEP_MIN_CELLS) B->sweep_zk[l] = rbgs_sweep_zk(int(gl.size()), gl.data());
+        if (sweeps && cells >= sweep_from(o.fused)) B->sweep_zk[l] = rbgs_sweep_zk(int(gl.size()), gl.data());
         const int szk = B->sweep_zk[l];
         B->rb[l].off = int(work.size());
         for (int b = 0; b < nbox; b++)
@@ -270,6 +270,7 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
     B->g_nu1 = o.nu1;
     B->g_nu2 = o.nu2;
     B->g_bot = o.bottom_iters;
+    B->g_fused = o.fused;  // the work lists hold its choice
     *st = MX_OK;
     return B;
 }
@@ -399,7 +400,7 @@ extern "C" mx_status mx_mac_project_batched(mx_ctx *c, int nbox, const mx_geom *
     }
     if (cudaSetDevice(c->device) != cudaSuccess) return set_err(c, MX_ERR_CUDA, "cudaSetDevice failed");
     if (!same_geoms(c->batch, nbox, g.data()) || c->batch->g_nu1 != o.nu1 || c->batch->g_nu2 != o.nu2 ||
-        c->batch->g_bot != o.bottom_iters) {
+        c->batch->g_bot != o.bottom_iters || c->batch->g_fused != o.fused) {
         destroy_batch_plan(c);
         c->batch = build_batch(c, nbox, g.data(), o, &st);
         if (!c->batch) return st;

@@ -1046,7 +1046,7 @@ struct CompPlan {
     // the refinement loop's graph and what it was captured with
     cudaGraphExec_t graph = nullptr;
     const void *k_part = nullptr;
-    int k_nu1 = -1, k_nu2 = -1, k_bot = -1, k_zcap = -1;
+    int k_nu1 = -1, k_nu2 = -1, k_bot = -1, k_zcap = -1, k_fused = -1;
     ~CompPlan() {
         if (graph) cudaGraphExecDestroy(graph);
         if (mem) cudaFree(mem);
@@ -1141,11 +1141,11 @@ void comp_body(cudaStream_t s, mx_ctx *c, CompPlan &P, double *phi_c, double *ph
     SolveState *dst = c->state;
     double *part = c->partials;
     comp_coarse_rhs_kernel<<<nbc, 256, 0, s>>>(G, P.rcb, P.rfb, dst, HC.lev[0].f);
-    vcycle(s, HC, o.nu1, o.nu2, o.bottom_iters, P.singular, nullptr, 0, zcap);
+    vcycle(s, HC, o.nu1, o.nu2, o.bottom_iters, P.singular, nullptr, o.fused, zcap);
     comp_coarse_update_kernel<<<nb, 256, 0, s>>>(G, phi_c, phi_f, HC.lev[0].e, dst, nbc);
     k_resid_fine(s, G, P.B, phi_c, phi_f, P.ff, P.rfb, nullptr);
     comp_fine_rhs_kernel<<<nbf, 256, 0, s>>>(Nf, P.rfb, dst, HF.lev[0].f);
-    vcycle(s, HF, o.nu1, o.nu2, o.bottom_iters, 0, nullptr, 0, zcap);
+    vcycle(s, HF, o.nu1, o.nu2, o.bottom_iters, 0, nullptr, o.fused, zcap);
     comp_fine_update_kernel<<<nbf, 256, 0, s>>>(Nf, phi_f, HF.lev[0].e, dst);
     k_resid_coarse(s, G, P.B, phi_c, phi_f, P.fc, P.rcb, part);
     k_resid_fine(s, G, P.B, phi_c, phi_f, P.ff, P.rfb, part);
@@ -1245,7 +1245,8 @@ extern "C" mx_status mx_mac_project_composite(mx_ctx *c, const mx_geom *geom, co
     MX_CUDA(c, cudaStreamSynchronize(s));
     if (!c->hstate->done) {
         if (o.use_graph) {
-            if (!P.graph || P.k_part != part || P.k_nu1 != o.nu1 || P.k_nu2 != o.nu2 || P.k_bot != o.bottom_iters || P.k_zcap != zcap) {
+            if (!P.graph || P.k_part != part || P.k_nu1 != o.nu1 || P.k_nu2 != o.nu2 || P.k_bot != o.bottom_iters ||
+                P.k_zcap != zcap || P.k_fused != o.fused) {
                 if (P.graph) {
                     cudaGraphExecDestroy(P.graph);
                     P.graph = nullptr;
@@ -1257,6 +1258,7 @@ extern "C" mx_status mx_mac_project_composite(mx_ctx *c, const mx_geom *geom, co
                 P.k_nu2 = o.nu2;
                 P.k_bot = o.bottom_iters;
                 P.k_zcap = zcap;
+                P.k_fused = o.fused;
             }
             MX_CUDA(c, cudaGraphLaunch(P.graph, s));
         } else {

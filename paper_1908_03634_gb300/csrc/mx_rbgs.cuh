@@ -2,6 +2,8 @@
 // with the two-pass colour kernels.
 #pragma once
 
+#include <climits>
+
 #include "mx_stencil.cuh"
 
 enum { RB_PLAIN = 0, RB_ZERO = 1, RB_PROLONG = 2 };
@@ -59,6 +61,13 @@ __device__ __forceinline__ float gs_update(const float b[6], const float v[6], f
 // 126 MB L2: measured, 256^3 96 us a sweep against 112 us, 160x192x224 42 against
 // 46, and 128^3, out of L2, 21 against 18.
 constexpr long long SWEEP_MIN_CELLS = 6LL << 20;
+
+// With mx_opts.fused = 1 they do from so many.
+constexpr long long FUSED_MIN_CELLS = 1LL << 18;
+// The cells from which a level smooths by sweeps under mx_opts.fused (2: none does).
+inline long long sweep_from(int fused) {
+    return fused == 2 ? LLONG_MAX : (fused ? FUSED_MIN_CELLS : SWEEP_MIN_CELLS);
+}
 
 // Whether the single-pass sweep supports this level (n_x a multiple of 4, at least 32).
 bool rbgs_fused_ok(const DGeom &g);

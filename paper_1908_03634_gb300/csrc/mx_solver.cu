@@ -186,16 +186,13 @@ void destroy_plans(mx_ctx *c) {
 // V-cycle on the correction equation L e = r (level-0 f holds r, e is zeroed here)
 
 // V-cycle on the correction equation L e = r (level-0 f holds r).
-//  * FP32 levels of >= SWEEP_MIN_CELLS cells (with fused = 1, of >=
-//    FUSED_MIN_CELLS): single-pass sweeps
+//  * FP32 levels of >= sweep_from(fused) cells: single-pass sweeps
 //    ping-ponging between e and e2; the first pre-sweep starts from e = 0
 //    without reading it and the first post-sweep applies the prolongation on
 //    load; the first output buffer is chosen so that the result ends in e;
 //  * other levels above the coarse end: two-pass colour kernels in place;
 //  * the coarse end (the levels that fit one cluster's shared memory, down to the
 //    bottom): one launch; without such a level, a BiCGStab bottom kernel.
-constexpr long long FUSED_MIN_CELLS = 1LL << 18;
-
 template <typename T>
 int coarse_start(const Hier<T> &H, int clustered) {
     for (int l = 0; l < H.nlev; l++)
@@ -210,7 +207,9 @@ void vcycle(cudaStream_t s, Hier<T> &H, int nu1, int nu2, int bot_iters, int sin
     const int lc = coarse_start(H, 1);
     const int ldown = lc < nl ? lc : nl - 1;  // levels with their own kernels
     const bool can_fuse = sizeof(T) == sizeof(float) && nu1 >= 1 && nu2 >= 1;
-    auto is_fused = [&](int l) { return can_fuse && H.lev[l].g.N >= (fused ? FUSED_MIN_CELLS : SWEEP_MIN_CELLS) && rbgs_fused_ok(H.lev[l].g); };
+    auto is_fused = [&](int l) {
+        return can_fuse && H.lev[l].g.N >= sweep_from(fused) && rbgs_fused_ok(H.lev[l].g);
+    };
     T *cur[MX_MAXLEV];
     for (int l = 0; l < ldown; l++) {
         Level<T> &L = H.lev[l];

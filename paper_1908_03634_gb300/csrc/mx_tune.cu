@@ -4,7 +4,7 @@
 // mx_autotune times whole solves of the caller's inputs on scratch copies of
 // U and phi, changing one setting at a time from the base options: the sweep
 // counts (nu1, nu2), then the z-depth of the stencil tiles (tile_z), then (MAC,
-// mixed precision) the single-pass sweep, or (nodal) the Chebyshev smoother
+// mixed precision) the levels smoothed by single-pass sweeps, or (nodal) the Chebyshev smoother
 // with its own degree candidates.  A change is kept when the solve
 // converges and its CUDA-event time (second of two calls: the first one builds
 // the plan and the loop graph) beats the best so far.  The winner is stored in
@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "mx_internal.cuh"
+#include "mx_rbgs.cuh"
 
 namespace {
 
@@ -231,11 +232,23 @@ extern "C" mx_status mx_autotune(mx_ctx *c, int op, const mx_geom *geom, const d
             if ((st = consider(cand))) break;
         }
     }
-    // 3. single-pass sweeps (MAC, FP32 V-cycles only)
+    // 3. on how many levels the single-pass sweeps smooth (MAC, FP32 V-cycles only):
+    // the values of `fused` that differ there
     if (!st && have && op == MX_OP_MAC && o.prec == MX_PREC_MIXED) {
-        mx_opts cand = cur;
-        cand.fused = cur.fused ? 0 : 1;
-        st = consider(cand);
+        DGeom gs[MX_MAXLEV];
+        const int nl = mac_levels(make_dgeom(geom), gs);
+        const auto swept = [&](int fused) {
+            return std::count_if(gs, gs + nl, [&](const DGeom &g) { return g.N >= sweep_from(fused) && rbgs_fused_ok(g); });
+        };
+        const mx_opts at = cur;
+        for (int f = 0; f < 3; f++) {
+            bool seen = swept(f) == swept(at.fused);
+            for (int e = 0; e < f; e++) seen = seen || swept(f) == swept(e);
+            if (seen) continue;
+            mx_opts cand = at;
+            cand.fused = f;
+            if ((st = consider(cand))) break;
+        }
     }
     // 3'. the Chebyshev smoother (nodal) at the chosen tile depth: a step is one
     // pass over the nodes where a colour sweep is four, so its degrees run higher

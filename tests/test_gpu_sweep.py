@@ -110,3 +110,62 @@ def test_restriction_by_columns_equals_one_cell_per_thread(mx, ctx):
         one = torch.zeros_like(rho[b])
         mx.mx_mac_project(ctx, g, *[cuda(t.numpy()) for t in us[b]], rho[b], beta0[b], sbar[b], one, opts, allow=allow)
         assert torch.equal(one, phi[b]), boxes[b]
+
+
+def big_problem(mx, n, bc, seed):
+    g = W.Geom(n, 1.0 / n[0], bc, bc)
+    gen = torch.Generator(device=DEV).manual_seed(seed)
+    rand = lambda s: torch.randn(s, dtype=torch.float64, device=DEV, generator=gen)
+    cs = mx.cell_shape(g)
+    rho, beta0 = torch.exp(0.5 * rand(cs)), torch.exp(0.5 * rand(cs))
+    return g, rho, beta0, rand(cs), [t.contiguous() for t in W._periodic_faces(g, [rand(g.face_shape(d)) for d in range(3)])]
+
+
+@pytest.mark.parametrize("n,bc", [((256, 256, 256), (P, P, N)), ((244, 200, 136), (D, P, N)), ((448, 126, 112), (N, D, P))])
+@pytest.mark.parametrize("nu", [(2, 3), (1, 1)])
+def test_sweeps_of_large_levels_equal_colour_passes(mx, ctx, n, bc, nu):
+    """fused = 0 on levels of 6 M cells and more, where the sweep is the default, and
+    fused = 1 on those below, against fused = 2: colour passes on every level."""
+    g, rho, beta0, sbar, u = big_problem(mx, n, bc, 8)
+    assert n[0] * n[1] * n[2] >= 6 << 20
+    out = []
+    for fused in (2, 0, 1):
+        phi = torch.zeros_like(rho)
+        st, info = mx.mx_mac_project(ctx, g, *[t.clone() for t in u], rho, beta0, sbar, phi,
+                                     mx.default_opts(fused=fused, nu1=nu[0], nu2=nu[1], max_outer=2),
+                                     allow=(mx.MX_OK, mx.MX_ERR_NOCONV))
+        assert info["vcycles"] == 2 and np.isfinite(info["rel_resid"])
+        out.append(phi)
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    mx.mx_profile_enable(ctx, True)
+    for fused, launches in ((2, 2 * nu[0] + 1 + 2 * nu[1]), (0, nu[0] + nu[1])):
+        mx.mx_profile_read(ctx)
+        mx.mx_mac_project(ctx, g, *[t.clone() for t in u], rho, beta0, sbar, torch.zeros_like(rho),
+                          mx.default_opts(fused=fused, nu1=nu[0], nu2=nu[1], max_outer=2), allow=(mx.MX_OK, mx.MX_ERR_NOCONV))
+        assert mx.mx_profile_read(ctx)["smooth_fine"][1] == 2 * launches
+    mx.mx_profile_enable(ctx, False)
+
+
+def test_batched_and_composite_calls_take_the_option(mx, ctx):
+    """The same bits from batches and composites whose levels sweep (fused = 1) and whose
+    levels do not (2)."""
+    boxes = [big_problem(mx, n, bc, 9) for n, bc in [((64, 48, 96), (P, P, N)), ((96, 40, 64), (D, N, P))]]
+    allow = (mx.MX_OK, mx.MX_ERR_NOCONV)
+    out = []
+    for fused in (2, 1, 0):
+        phi = [torch.zeros_like(b[1]) for b in boxes]
+        mx.mx_mac_project_batched(ctx, [b[0] for b in boxes], *[[b[4][d].clone() for b in boxes] for d in range(3)],
+                                  [b[1] for b in boxes], [b[2] for b in boxes], [b[3] for b in boxes], phi,
+                                  mx.default_opts(fused=fused, max_outer=2), allow=allow)
+        out.append(phi)
+    assert all(torch.equal(a, b) and torch.equal(a, c) for a, b, c in zip(*out))
+    coarse = big_problem(mx, (64, 64, 64), (P, P, N), 10)
+    fine = big_problem(mx, (64, 64, 64), (N, N, N), 11)
+    out = []
+    for fused in (2, 1, 0):
+        pc, pf = torch.zeros_like(coarse[1]), torch.zeros_like(fine[1])
+        mx.mx_mac_project_composite(ctx, coarse[0], (16, 16, 16), (48, 48, 48), [t.clone() for t in coarse[4]], *coarse[1:4],
+                                    pc, [t.clone() for t in fine[4]], *fine[1:4], pf,
+                                    mx.default_opts(fused=fused, max_outer=2), allow=allow)
+        out.append((pc, pf))
+    assert all(torch.equal(out[0][k], out[m][k]) for k in (0, 1) for m in (1, 2))
