@@ -56,3 +56,18 @@ def test_launch_count_without_a_mean_to_remove():
     per = _G((256, 256, 256), (0, 0, 1), (0, 0, 1))
     dir_ = _G((256, 256, 256), (0, 0, 2), (0, 0, 2))
     assert bench.launches_per_solve(per, _O(2, 3), 7, True) - bench.launches_per_solve(dir_, _O(2, 3), 7, True) == 2
+
+
+def test_launch_count_of_the_schedule_the_bench_runs():
+    # with the arguments the bench passes: 256^3 by sweeps (2 + 1 + 3 launches), 128^3 and
+    # 64^3 by colour passes (4 + 1 + 1 + 6), the coarse end from 32^3; with the coarse-end
+    # launch, update/residual, its finalize and the graph's condition kernel 6 + 24 + 4
+    # per V-cycle, and 15 + 6 launches around the loop
+    g = _G((256, 256, 256), (0, 0, 1), (0, 0, 1))
+    run = lambda fused, vc=7: bench.launches_per_solve(g, _O(2, 3, fused), vc, True, 0, bench.SWEEP_CELLS,
+                                                       bench.CLUSTER_CELLS)
+    assert run(0) == 259
+    assert run(0, 8) - run(0) == 34
+    # fused = 1: sweeps on 128^3 and 64^3 too; fused = 2: colour passes on every level
+    assert run(1, 8) - run(1) == 6 + 12 + 4
+    assert run(2, 8) - run(2) == 36 + 4
