@@ -304,7 +304,8 @@ __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &
     const int n = int(L.g.N), nx = L.g.n[0], ny = L.g.n[1], nz = L.g.n[2], nxy = nx * ny;
     T b[B][6], den[B], dinv[B], xv[B], r[B], r0[B] = {}, p[B], v[B];
     unsigned nb[B][3];
-    if (threadIdx.x < 2) scr[threadIdx.x * (n + 1) + n] = T(0);
+    const unsigned vec = unsigned(__cvta_generic_to_shared(scr));
+    if (threadIdx.x < 2) team_put(vec + (threadIdx.x * (n + 1) + n) * unsigned(sizeof(T)), T(0));
     T a[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
     for (int q = 0; q < B; q++) {
@@ -362,17 +363,19 @@ __device__ __forceinline__ void team_bicgstab(TeamShared<T> &S, const Level<T> &
             bool stop = false;
 #pragma unroll 1
             for (int h = 0; h < 2; h++) {  // y = L w: v = L p, then t = L s
-                T *e = scr + h * (n + 1);
+                const unsigned e = vec + h * (n + 1) * unsigned(sizeof(T));
+                const auto at = [&](unsigned c) { return team_get(e + c * unsigned(sizeof(T)), T(0)); };
 #pragma unroll
                 for (int q = 0; q < B; q++)
-                    if (int(threadIdx.x) + q * nthr < n) e[threadIdx.x + q * nthr] = rmul(w[q], dinv[q]);
+                    if (int(threadIdx.x) + q * nthr < n)
+                        team_put(e + (threadIdx.x + q * nthr) * unsigned(sizeof(T)), rmul(w[q], dinv[q]));
                 team.barrier();
                 a[0] = a[1] = a[2] = a[3] = T(0);
 #pragma unroll
                 for (int q = 0; q < B; q++) {
-                    const T s0 = rfma(b[q][0], e[nb[q][0] & 0xffffu], rmul(b[q][1], e[nb[q][0] >> 16]));
-                    const T s1 = rfma(b[q][2], e[nb[q][1] & 0xffffu], rmul(b[q][3], e[nb[q][1] >> 16]));
-                    const T s2 = rfma(b[q][4], e[nb[q][2] & 0xffffu], rmul(b[q][5], e[nb[q][2] >> 16]));
+                    const T s0 = rfma(b[q][0], at(nb[q][0] & 0xffffu), rmul(b[q][1], at(nb[q][0] >> 16)));
+                    const T s1 = rfma(b[q][2], at(nb[q][1] & 0xffffu), rmul(b[q][3], at(nb[q][1] >> 16)));
+                    const T s2 = rfma(b[q][4], at(nb[q][2] & 0xffffu), rmul(b[q][5], at(nb[q][2] >> 16)));
                     y[q] = rfma(-den[q], rmul(w[q], dinv[q]), radd(radd(s0, s1), s2));
                     a[0] = rfma(r0[q], y[q], a[0]);
                     a[1] = rfma(w[q], w[q], a[1]);
@@ -539,7 +542,6 @@ template <typename T, int SLMAX>
 __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &A, int rank) {
     constexpr int B = sizeof(T);
     __shared__ TeamShared<T> bottom;
-    if (threadIdx.x == 0 && rank == 0) team_init(bottom, max(32, bottom_threads(int(A.lev[A.nl - 1].L.g.N))));
     for (int q = threadIdx.x * B; q < A.roff; q += CT * B) sm_at<T>(q) = T(0);
     __syncthreads();
     const int first = rank * A.lev[0].pp, nxy0 = int(A.lev[0].L.g.nxy);  // this CTA's planes of the first level

@@ -697,8 +697,6 @@ __global__ void __launch_bounds__(NBT) nd_bottom_kernel(NLevel<T> L, T *scr, int
     if (n <= NBT) {
         __shared__ NdTeam<T> S;
         const int nthr = (n + 31) & ~31;
-        if (threadIdx.x == 0) team_init(S.team, nthr);
-        __syncthreads();
         if (int(threadIdx.x) < nthr) nd_team_bicgstab(S, L, iters, nthr);
         return;
     }

@@ -4,26 +4,15 @@
 
 #include "mx_internal.cuh"
 
-// What a team keeps in static shared memory: the partial sums and the mbarrier on
-// which one lane of each warp arrives.  (A named barrier counts a warp once for each
-// part in which it arrives, and after the sums' divergent branches that is up to the
-// compiler.)  The sums are stored and loaded by inline assembly that clobbers memory:
-// with plain accesses to the array one build of a bottom solve read the first warp's
-// sum and none of the others', whatever the barrier between.  A wait ends after 2^20
-// tries at the latest.
+// A team's partial sums.  All that its threads exchange between barriers, the vectors
+// of the solves too, goes through team_put and team_get, whose order against the barrier
+// is fixed in the source: with plain accesses to the static array a build of an
+// earlier solve read the first warp's sum and none of the others', for a reason
+// that was not found.
 template <typename T>
 struct TeamShared {
-    unsigned long long bar;
     T red[2][4][32];
 };
-
-// One thread, before a block barrier and any use: a team of nthr threads.
-template <typename T>
-__device__ __forceinline__ void team_init(TeamShared<T> &S, int nthr) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(unsigned(__cvta_generic_to_shared(&S.bar))),
-                 "r"(nthr >> 5)
-                 : "memory");
-}
 
 __device__ __forceinline__ void team_put(unsigned a, float v) {
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
@@ -49,31 +38,19 @@ __device__ __forceinline__ double team_get(unsigned a, double) {
 // between a call's reads and the writes of the next but one.
 template <typename T>
 struct TeamSum {
-    unsigned red, bar;  // shared addresses: two buffers of partial sums, the barrier
-    int nthr, turn = 0, phase = 0;
+    unsigned red;  // shared address of the two buffers of partial sums
+    int nthr, turn = 0;
 
     __device__ __forceinline__ TeamSum(TeamShared<T> &S, int n)
-        : red(unsigned(__cvta_generic_to_shared(&S.red[0][0][0]))),
-          bar(unsigned(__cvta_generic_to_shared(&S.bar))),
-          nthr(n) {}
+        : red(unsigned(__cvta_generic_to_shared(&S.red[0][0][0]))), nthr(n) {}
     __device__ __forceinline__ unsigned slot(int g, int w) const {
         return red + ((turn * 4 + g) * 32 + w) * unsigned(sizeof(T));
     }
+    // named barrier 1 of nthr threads, in the form that does not need a warp's threads
+    // to arrive together
     __device__ __forceinline__ void barrier() {
         __syncwarp();
-        if ((threadIdx.x & 31) == 0)
-            asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(bar) : "memory");
-        int ok = 0;
-#pragma unroll 1
-        for (int spin = 0; !ok && spin < (1 << 20); spin++)
-            asm volatile(
-                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                "selp.b32 %0, 1, 0, p;\n\t}"
-                : "=r"(ok)
-                : "r"(bar), "r"(phase)
-                : "memory");
-        __syncwarp();
-        phase ^= 1;
+        asm volatile("barrier.sync 1, %0;" ::"r"(nthr) : "memory");
     }
     static __device__ __forceinline__ T group_sum(T k) {
 #pragma unroll
