@@ -104,3 +104,98 @@ def test_largest_bottoms(mx, ctx, n, bc):
     mx.mx_mac_project_batched(ctx, [g], *[[cuda(t)] for t in u], [cuda(rho)], [cuda(beta0)], [cuda(sbar)], [phi],
                               mx.default_opts())
     assert np.array_equal(phi.cpu().numpy(), phis[1])
+
+
+def flux(g, b, x):
+    """sum over the faces of b times the neighbour's value (0 beyond a face without one)"""
+    out = np.zeros_like(x)
+    for d in range(3):
+        ax = 2 - d
+        n = x.shape[ax]
+        lo, hi = np.roll(x, 1, ax), np.roll(x, -1, ax)
+        if g.lo[d] != P:
+            np.moveaxis(lo, ax, 0)[0] = 0.0
+            np.moveaxis(hi, ax, 0)[-1] = 0.0
+        out += np.take(b[d], range(n), ax) * lo + np.take(b[d], range(1, n + 1), ax) * hi
+    return out
+
+
+def diagonal(b):
+    return sum(np.take(b[d], range(b[d].shape[2 - d] - 1), 2 - d) + np.take(b[d], range(1, b[d].shape[2 - d]), 2 - d)
+               for d in range(3))
+
+
+def vcycle(g, b, f, h, nu):
+    """One V-cycle on L e = f in FP64 with an exact bottom solve, and the bound 1e-4 of
+    the bottom residual's norm puts on the bottom's error."""
+    n = f.shape
+    den = diagonal(b)
+    if any(k % 2 or k < 4 for k in n):
+        m = np.empty((f.size, f.size))
+        for c in range(f.size):
+            unit = np.zeros(f.size)
+            unit[c] = 1.0
+            unit = unit.reshape(n)
+            m[:, c] = (flux(g, b, unit) - den * unit).ravel() / h**2
+        free = f - f.mean() if O.singular(g) else f
+        s = np.linalg.svd(m, compute_uv=False)
+        least = s[s > 1e-9 * s[0]].min()
+        e = np.linalg.lstsq(m, free.ravel(), rcond=1e-9)[0].reshape(n)
+        return e - (e.mean() if O.singular(g) else 0.0), 1e-4 * np.linalg.norm(free) / least
+    colour = np.indices(n).sum(axis=0) % 2
+    e = np.zeros(n)
+
+    def smooth():
+        for _ in range(nu):
+            for c in (0, 1):
+                e[colour == c] = ((flux(g, b, e) - h**2 * f) / den)[colour == c]
+
+    smooth()
+    r = f - (flux(g, b, e) - den * e) / h**2
+    pairs = lambda a: a.reshape(n[0] // 2, 2, n[1] // 2, 2, n[2] // 2, 2)
+    bc = [0.25 * sum(b[0][i::2, j::2, ::2] for i in (0, 1) for j in (0, 1)),
+          0.25 * sum(b[1][i::2, ::2, j::2] for i in (0, 1) for j in (0, 1)),
+          0.25 * sum(b[2][::2, i::2, j::2] for i in (0, 1) for j in (0, 1))]
+    ec, bound = vcycle(g, bc, pairs(r).mean(axis=(1, 3, 5)), 2 * h, nu)
+    pairs(e)[...] += ec[:, None, :, None, :, None]
+    smooth()
+    return e, bound
+
+
+@pytest.mark.parametrize("n,bc", [((4, 4, 4), (N, P, P)), ((8, 12, 20), (P, D, N)), ((16, 16, 16), (P, P, P)),
+                                  ((20, 24, 28), (P, P, N)), ((36, 28, 20), (D, D, D)), ((32, 32, 32), (N, N, P)),
+                                  ((64, 16, 12), (P, P, N))])
+@pytest.mark.parametrize("nu", [1, 2])
+def test_one_fp64_vcycle(mx, ctx, n, bc, nu):
+    """phi after one FP64 V-cycle against the same cycle in numpy with an exact bottom
+    solve.  The bottom's error is at most 1e-4 of its right-hand side's norm over the
+    least singular value; prolongation copies it and the smoother's rows are averages, so
+    no value of phi is off by more, beyond rounding (1e-11 of max |phi|)."""
+    g, rho, beta0, sbar, u = problem(n, bc)
+    f, b = O.mac_rhs(g, u, beta0, sbar)[0], O.mac_coeffs(g, rho, beta0)
+    for d in range(3):  # half a cell from the centre to a Dirichlet face
+        for side, at in ((g.lo[d], 0), (g.hi[d], -1)):
+            if side == D:
+                np.moveaxis(b[d], 2 - d, 0)[at] *= 2.0
+    want, bound = vcycle(g, b, f, g.dx, nu)
+    want -= want.mean() if O.singular(g) else 0.0
+    phi = torch.zeros(O.cell_shape(g), dtype=torch.float64, device=DEV)
+    mx.mx_mac_project(ctx, g, *[cuda(t) for t in u], cuda(rho), cuda(beta0), cuda(sbar), phi,
+                      mx.default_opts(prec=0, nu1=nu, nu2=nu, max_outer=1), allow=(mx.MX_OK, mx.MX_ERR_NOCONV))
+    off = np.abs(phi.cpu().numpy() - want).max()
+    assert bound <= 0.1 * np.abs(want).max()  # or the comparison would say little
+    assert off <= (2 if O.singular(g) else 1) * bound + 1e-11 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("n", [(1, 1, 2), (3, 5, 7), (3, 5, 17), (9, 7, 15), (15, 13, 17), (17, 17, 17)])
+@pytest.mark.parametrize("bc", [(N, N, N), (N, D, N)])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_bottom_solve_alone(mx, ctx, n, bc, prec):
+    """Boxes of one level: a V-cycle is the bottom solve, in each of its forms, to 1e-4 of
+    the right-hand side's 2-norm, so at most 1e-4 sqrt(cells) of its maximum; the same
+    again for the rounding of the iterates."""
+    g, rho, beta0, sbar, u = problem(n, bc)
+    phi = torch.zeros(O.cell_shape(g), dtype=torch.float64, device=DEV)
+    st, info = mx.mx_mac_project(ctx, g, *[cuda(t) for t in u], cuda(rho), cuda(beta0), cuda(sbar), phi,
+                                 mx.default_opts(prec=prec, max_outer=1), allow=(mx.MX_OK, mx.MX_ERR_NOCONV))
+    assert info["vcycles"] <= 1 and info["rel_resid"] <= 2e-4 * np.sqrt(phi.numel())
