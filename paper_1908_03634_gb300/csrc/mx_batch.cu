@@ -131,6 +131,10 @@ static BatchPlan *build_batch(mx_ctx *c, int nbox, const DGeom *g, const mx_opts
                 cells += gl.back().N;
                 sweeps = sweeps && rbgs_fused_ok(gl.back());
             }
+        // sweeps as on a single level of as many cells, whatever the boxes' extents: though
+        // tiles of short rows are half halo, a V-cycle (colour passes, sweeps) of 200 boxes
+        // of 32^3 took 0.867 and 0.590 ms, 96 of 48^3 1.140 and 0.893, 48 of 64^3 1.125 and
+        // 1.018, 96 of 64x32x48 0.838 and 0.799, 16 of 104^3 1.897 and 1.506
         if (sweeps && cells >= sweep_from(o.fused)) B->sweep_zk[l] = rbgs_sweep_zk(int(gl.size()), gl.data());
         const int szk = B->sweep_zk[l];
         B->rb[l].off = int(work.size());

@@ -32,7 +32,8 @@ struct DGeom {
 __host__ __device__ inline bool gper(const DGeom &g, int d) { return g.lo[d] == MX_BC_PERIODIC; }
 
 // FP64 levels keep the reciprocal of each cell's coefficient sum (the FP64
-// division takes eleven FMAs' time); FP32 divides as it goes.
+// division takes eleven FMAs' time); FP32 takes the hardware's approximate
+// reciprocal as it goes.
 template <typename T>
 struct LevelInverse {};
 template <>
@@ -269,8 +270,10 @@ dim3 resid_restrict_fine_grid(const DGeom &fine, int zcf, bool quad);
 // by 2 x 2 columns per thread where the level allows it; smaller ones need the four
 // times as many threads of one cell each.  Whole solves of 8 cycles, columns against
 // cells: 32x192x192 2.06 against 2.08 ms, 104^3 4.33 against 4.36, 128^3 2.16 against
-// 2.20, 160x32x208 1.79 against 1.81.  Single boxes of rows under 32 cells, which would
-// leave most of a warp idle, keep one cell per thread.
+// 2.20, 160x32x208 1.79 against 1.81.  Batches have no bound on the row: a V-cycle of
+// 16 boxes of 8x128x128 took 0.930 ms by columns and 0.942 by cells, 120 of 24^3 0.282 and
+// 0.292, 70 of 28^3 0.284 and 0.290.  Single boxes of rows under 32 cells keep one cell
+// per thread (not measured).
 constexpr long long RESTRICT_QUAD_MIN = 1LL << 20;
 bool resid_restrict_quad_ok(const Level<float> &fine);
 // fine: the descriptors whose e is corrected (levs, or those with e and e2 exchanged)
